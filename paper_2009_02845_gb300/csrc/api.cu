@@ -85,6 +85,10 @@ int64_t srht_pad(int64_t K) {
     return p;
 }
 
+// Row stride of a dense matrix of n columns: 16-byte rows, so that a matrix of any size can
+// be copied by TMA (very narrow ones are kept packed).  The columns past n are zero.
+int64_t row_stride(int64_t n) { return n < 32 ? n : ceil_div(n, 4) * 4; }
+
 int kp_bucket(int k) { return k <= 16 ? 16 : (k <= 32 ? 32 : (k <= 64 ? 64 : 128)); }
 
 constexpr int MAX_SPLITS = 32;
@@ -111,6 +115,7 @@ struct dsanls_ctx {
     bool has_dense = false, has_sparse = false;
     bool sumsq_dirty = false;  // ||M||^2 of new dense data not computed yet (done when needed)
     float *M = nullptr, *MT = nullptr;
+    int64_t ldM = 0, ldT = 0;  // row strides of M (>= n) and M^T (>= m): whole 16 bytes for TMA
     __nv_bfloat16 *Mb = nullptr, *MTb = nullptr;
     // FP32 form on tensor cores: three-way bf16 splits of M and M^T
     __nv_bfloat16 *M3[3] = {nullptr, nullptr, nullptr}, *MT3[3] = {nullptr, nullptr, nullptr};
@@ -127,13 +132,16 @@ struct dsanls_ctx {
     __nv_bfloat16 *U16 = nullptr, *V16 = nullptr;
 
     // workspaces (sized by prepare())
-    int64_t cfg_key[7] = {-1, -1, -1, -1, -1, -1, -1};
+    int64_t cfg_key[8] = {-1, -1, -1, -1, -1, -1, -1, -1};
     float *S = nullptr;
     __nv_bfloat16 *Sb = nullptr;
     int32_t *J = nullptr;
     float *A = nullptr;
     float *W = nullptr;
     float *Wpart = nullptr;
+    // split products (FP32, projected gradient): split-K partials, second operand's parts
+    float *Gpart = nullptr;
+    __nv_bfloat16 *Gparts = nullptr;
     float *R = nullptr;
     float *Rpart = nullptr;
     __nv_bfloat16 *Ytb = nullptr;  // bf16 Y^T (k x K) for the tensor-core B = Y^T S
@@ -251,11 +259,51 @@ void factors_to_f32(dsanls_ctx *h, cudaStream_t s) {
     launch_cast_f32(h->V16, h->n * h->k, h->V, s);
 }
 
-// The FP32 form of a dense-sketch product runs on tensor cores from three-way
-// bf16 splits when the rows of both orientations of M are 16-byte multiples
-// (TMA), else on CUDA cores.
+// Alg. 3's sweep multiplies a rounding difference of R by 1e2 and more (a step of 100
+// columns in binary32 is 4e-5 off 64 bits with R exact to 1e-7), so its products keep
+// one binary32 FMA chain per output; the projected-gradient step takes the split
+// products on tensor cores, which are no further from 64 bits than the chain.
+bool chained(const dsanls_ctx *h) { return h->opt.solver == DSANLS_SOLVER_RCD; }
+
+// FP32 form, dense sketch: A = X S (and with Alg. 3 also R = X P) from split copies of M and
+// M^T when the rows of both are 16-byte multiples in bf16 (TMA).  256 columns of S share a
+// copied tile of X there (244 TFLOP/s of binary32 work; the split on the fly, 128 columns
+// a tile, 215); the narrow R = X P reads 6 bytes per entry of X that way and 4 as binary32.
 bool fp32_split(const dsanls_ctx *h) {
-    return h->has_dense && h->opt.precision == DSANLS_PREC_FP32 && h->m % 8 == 0 && h->n % 8 == 0;
+    return h->has_dense && h->opt.precision == DSANLS_PREC_FP32 && dense_kind(h->sketch) &&
+           (h->opt.order == DSANLS_ORDER_PAPER || chained(h)) && h->m % 8 == 0 && h->n % 8 == 0;
+}
+
+// workspace of a half-step's split products: floats of partial sums and bf16 elements of
+// second operands' parts
+struct SplitNeed {
+    int64_t part = 0, parts = 0;
+};
+SplitNeed split_need(const dsanls_ctx *h) {
+    SplitNeed need;
+    for (int side = 0; side < 2; ++side) {
+        const int64_t rows = side == 0 ? h->m : h->n, K = side == 0 ? h->n : h->m, k = h->k;
+        const int64_t dd = side == 0 ? h->d : d_v_of(h);
+        auto use = [&](int64_t M, int64_t N, int64_t L) {
+            need.part = std::max(need.part, split_gemm_plan(M, N, L).part_elems);
+            need.parts = std::max(need.parts, 3 * N * split_parts_ld(L));
+        };
+        if (h->sketch == DSANLS_SKETCH_SUBSAMPLE) {
+            if (h->has_dense) use(rows, k, dd);
+        } else if (h->sketch == DSANLS_SKETCH_IDENTITY) {
+            if (h->has_dense) use(rows, k, K);
+        } else {
+            use(dd, k, K);
+            if (h->opt.order == DSANLS_ORDER_REASSOCIATED) {
+                use(K, k, dd);
+                if (h->has_dense) use(rows, k, K);
+            } else {
+                use(rows, k, dd);
+                if (h->has_dense && !fp32_split(h)) use(rows, dd, K);
+            }
+        }
+    }
+    return need;
 }
 
 // Sum of the d largest row lengths of a CSR row pointer (the most entries a
@@ -273,9 +321,9 @@ int64_t top_sum(const std::vector<int64_t> &ptr, int64_t d) {
 // (Re)allocate the per-configuration workspaces.
 void prepare(dsanls_ctx *h) {
     const int dv = d_v_of(h);
-    const int64_t key[7] = {h->sketch, h->d, dv, h->opt.precision, h->has_dense ? 1 : 0, h->has_sparse ? 1 : 0,
-                            h->opt.order};
-    if (std::equal(key, key + 7, h->cfg_key)) return;
+    const int64_t key[8] = {h->sketch, h->d, dv, h->opt.precision, h->has_dense ? 1 : 0, h->has_sparse ? 1 : 0,
+                            h->opt.order, chained(h) ? 1 : 0};
+    if (std::equal(key, key + 8, h->cfg_key)) return;
     invalidate_graph(h);
     const int64_t m = h->m, n = h->n, k = h->k;
     const int64_t dmax = std::max<int64_t>(h->d, dv);
@@ -316,7 +364,10 @@ void prepare(dsanls_ctx *h) {
                                        (int64_t)1})
                            : 0);
     dalloc(h->W, k * (ident ? std::max(m, n) : dmax));
-    dalloc(h->Wpart, (gauss && !bf16) ? (int64_t)MAX_SPLITS * k * dmax : 0);
+    dalloc(h->Wpart, (gauss && !bf16 && chained(h)) ? (int64_t)MAX_SPLITS * k * dmax : 0);
+    const SplitNeed need = (!bf16 && !chained(h)) ? split_need(h) : SplitNeed{};
+    dalloc(h->Gpart, need.part);
+    dalloc(h->Gparts, need.parts);
     dalloc(h->Ytb, ((gauss && bf16) || ident_tc) ? k * std::max(m, n) : 0);
     dalloc(h->Bpart, (gauss && bf16) ? tc_gemm_part_elems(k, dmax) : 0);
     dalloc(h->R, std::max(m, n) * k);
@@ -345,7 +396,7 @@ void prepare(dsanls_ctx *h) {
         h->sub[0].release();
         h->sub[1].release();
     }
-    std::copy(key, key + 7, h->cfg_key);
+    std::copy(key, key + 8, h->cfg_key);
 }
 
 // ---------------------------------------------------------------------------
@@ -370,6 +421,7 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
     // data views: X = rows x K (M or M^T), XT = K x rows
     const float *X = side == 0 ? h->M : h->MT;
     const float *XT = side == 0 ? h->MT : h->M;
+    const int64_t ldX = side == 0 ? h->ldM : h->ldT, ldXT = side == 0 ? h->ldT : h->ldM;
     const int64_t *xp = side == 0 ? h->rp : h->trp;
     const int32_t *xc = side == 0 ? h->ci : h->tci;
     const float *xv = side == 0 ? h->cv : h->tcv;
@@ -390,6 +442,18 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
                          h->Gf, kp, h->aux_stream);
         DSANLS_CUDA(cudaEventRecord(h->ev_join, h->aux_stream));
         forked = true;
+    };
+
+    // one of the FP32 form's products (c_trans: stored transposed, split products only)
+    auto product = [&](const GemmArgs &g, bool c_trans = false) {
+        if (chained(h)) {
+            launch_sgemm(g, s);
+            return;
+        }
+        launch_split_parts(g.B, g.ldb, g.b_kcontig, g.gb, g.N, g.K, h->Gparts, s);
+        launch_split_gemm(SplitGemm{g.M, g.N, g.K, g.A, g.lda, g.a_kcontig, g.ga, h->Gparts, 3, g.C, g.ldc, c_trans,
+                                    g.alpha, h->Gpart},
+                          h->flag, s);
     };
 
     mark(pe, DSANLS_PHASE_SKETCH, s);
@@ -434,6 +498,14 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
             // B = Y^T S (k x dd) on tensor cores from bf16 Y^T and S^T, split-K
             launch_transpose_bf16(Y, K, k, h->Ytb, s);
             launch_tc_gemm(h->Ytb, h->Sb, k, K, dd, h->Bpart, h->W, h->flag, s);
+        } else if (!chained(h)) {
+            // B^T = S^T Y (dd x k) on tensor cores, stored transposed
+            GemmArgs g{};
+            g.M = dd; g.N = k; g.K = K;
+            g.A = h->S; g.lda = dd; g.a_kcontig = false;
+            g.B = Y; g.ldb = k; g.b_kcontig = false;
+            g.C = h->W; g.ldc = dd; g.alpha = 1.0f;
+            product(g, true);
         } else {
             // B = Y^T S  (k x dd), split over K, partials summed in order
             const int64_t tiles = ceil_div(k, 128) * ceil_div(dd, 128);
@@ -465,7 +537,7 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
                 g.A = h->S; g.lda = dd; g.a_kcontig = true;
                 g.B = h->W; g.ldb = dd; g.b_kcontig = true;
                 g.C = h->P; g.ldc = k; g.alpha = 1.0f; g.splits = 1;
-                launch_sgemm(g, s);
+                product(g);
             }
             mark(pe, DSANLS_PHASE_RHS, s);
             if (fp8) {
@@ -480,10 +552,10 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
             } else if (dense) {
                 GemmArgs g{};
                 g.M = rows; g.N = k; g.K = K;
-                g.A = X; g.lda = K; g.a_kcontig = true;
+                g.A = X; g.lda = ldX; g.a_kcontig = true;
                 g.B = h->P; g.ldb = k; g.b_kcontig = false;
                 g.C = h->R; g.ldc = k; g.alpha = 1.0f; g.splits = 1;
-                launch_sgemm(g, s);
+                product(g);
             } else {
                 launch_spmm_rows(xp, xc, xv, rows, h->P, K, k, k, 1.0f, h->R, k, s);
             }
@@ -507,10 +579,10 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
             } else if (dense) {
                 GemmArgs g{};
                 g.M = rows; g.N = dd; g.K = K;
-                g.A = X; g.lda = K; g.a_kcontig = true;
+                g.A = X; g.lda = ldX; g.a_kcontig = true;
                 g.B = h->S; g.ldb = dd; g.b_kcontig = false;
                 g.C = h->A; g.ldc = dd; g.alpha = 1.0f; g.splits = 1;
-                launch_sgemm(g, s);
+                product(g);
             } else {
                 launch_spmm_rows(xp, xc, xv, rows, h->S, K, dd, dd, 1.0f, h->A, dd, s);
             }
@@ -520,7 +592,7 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
             g.A = h->A; g.lda = dd; g.a_kcontig = true;
             g.B = h->W; g.ldb = dd; g.b_kcontig = true;
             g.C = h->R; g.ldc = k; g.alpha = 1.0f; g.splits = 1;
-            launch_sgemm(g, s);
+            product(g);
         }
     } else if (h->sketch == DSANLS_SKETCH_SUBSAMPLE) {
         const float c = (float)std::sqrt((double)K / (double)dd);
@@ -542,11 +614,11 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
         if (dense) {
             GemmArgs g{};
             g.M = rows; g.N = k; g.K = dd;
-            g.A = XT; g.lda = rows; g.ga = h->J; g.a_kcontig = false;
+            g.A = XT; g.lda = ldXT; g.ga = h->J; g.a_kcontig = false;
             g.B = Y; g.ldb = k; g.gb = h->J; g.b_kcontig = false;
             g.C = h->R; g.ldc = k; g.alpha = c2; g.splits = 1;
             mark(pe, DSANLS_PHASE_RHS, s);
-            launch_sgemm(g, s);
+            product(g);
         } else {
             // X[:, J] gathered from the rows J of the CSR of X^T, then
             // R = c^2 X[:, J] Y[J, :] row by row
@@ -580,10 +652,10 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
         } else if (dense) {
             GemmArgs g{};
             g.M = rows; g.N = k; g.K = K;
-            g.A = X; g.lda = K; g.a_kcontig = true;
+            g.A = X; g.lda = ldX; g.a_kcontig = true;
             g.B = Y; g.ldb = k; g.b_kcontig = false;
             g.C = h->R; g.ldc = k; g.alpha = 1.0f; g.splits = 1;
-            launch_sgemm(g, s);
+            product(g);
         } else {
             launch_spmm_rows(xp, xc, xv, rows, Y, K, k, k, 1.0f, h->R, k, s);
         }
@@ -675,7 +747,7 @@ void copy_in(void *dst, const void *src, size_t bytes, int on_device, cudaStream
 // ||M||^2 into dscal[0] when the dense data changed since it was last computed
 void ensure_sumsq(dsanls_ctx *h) {
     if (!h->sumsq_dirty || !h->has_dense) return;
-    launch_sumsq(h->M, h->m * h->n, h->work, WORK_ELEMS, h->dscal + 0, h->stream());
+    launch_sumsq(h->M, h->m * h->ldM, h->work, WORK_ELEMS, h->dscal + 0, h->stream());
     h->sumsq_dirty = false;
 }
 
@@ -715,6 +787,7 @@ void prime_kernel_attributes() {
     prime_rng_attributes(max_smem);
     prime_solver_attributes(max_smem);
     prime_tc_attributes(max_smem);
+    prime_split_gemm_attributes(max_smem);
     batch_prime_tc(max_smem);
     done[dev] = true;
 }
@@ -759,6 +832,8 @@ int dsanls_create(int64_t m, int64_t n, int32_t k, int32_t d, int32_t sketch_kin
     } catch (...) {
         return DSANLS_ENOMEM;
     }
+    h->ldM = row_stride(n);
+    h->ldT = row_stride(m);
     h->m = m; h->n = n; h->k = k; h->d = d; h->sketch = sketch_kind; h->seed = seed;
     dsanls_default_options(&h->opt);
     if (sketch_kind == DSANLS_SKETCH_IDENTITY) h->opt.d_v = (int32_t)m;
@@ -883,14 +958,20 @@ int dsanls_set_dense(dsanls_t h, const float *M, int64_t ld, int32_t on_device) 
         }
         // new values in the buffers of earlier dense data keep the captured graph valid
         const bool refresh = h->has_dense && h->M && h->MT;
-        if (!h->M) dalloc(h->M, h->m * h->n);
-        if (!h->MT) dalloc(h->MT, h->m * h->n);
+        if (!h->M) {
+            dalloc(h->M, h->m * h->ldM);
+            if (h->ldM > h->n) DSANLS_CUDA(cudaMemsetAsync(h->M, 0, (size_t)(h->m * h->ldM) * sizeof(float), s));
+        }
+        if (!h->MT) {
+            dalloc(h->MT, h->n * h->ldT);
+            if (h->ldT > h->m) DSANLS_CUDA(cudaMemsetAsync(h->MT, 0, (size_t)(h->n * h->ldT) * sizeof(float), s));
+        }
         const bool bf16 = h->opt.precision == DSANLS_PREC_BF16, fp8 = h->opt.precision == DSANLS_PREC_FP8;
         const bool cast_b = refresh && bf16 && h->Mb;
         if (on_device) {
-            DSANLS_CUDA(cudaMemcpy2DAsync(h->M, h->n * sizeof(float), M, ld * sizeof(float), h->n * sizeof(float),
+            DSANLS_CUDA(cudaMemcpy2DAsync(h->M, h->ldM * sizeof(float), M, ld * sizeof(float), h->n * sizeof(float),
                                           h->m, cudaMemcpyDeviceToDevice, s));
-            launch_transpose(h->M, h->n, h->m, h->n, h->MT, h->m, s);
+            launch_transpose(h->M, h->ldM, h->m, h->n, h->MT, h->ldT, s);
             if (cast_b) launch_copy_cast_bf16(h->M, h->m * h->n, h->Mb, s);
         } else {
             // host data: copied in chunks of rows (about 256 MB); the transpose (and bf16
@@ -898,11 +979,11 @@ int dsanls_set_dense(dsanls_t h, const float *M, int64_t ld, int32_t on_device) 
             const int64_t ch = std::max<int64_t>(1024, ((int64_t)256 << 20) / (h->n * (int64_t)sizeof(float)));
             for (int64_t r0 = 0; r0 < h->m; r0 += ch) {
                 const int64_t rc = std::min(ch, h->m - r0);
-                DSANLS_CUDA(cudaMemcpy2DAsync(h->M + r0 * h->n, h->n * sizeof(float), M + r0 * ld, ld * sizeof(float),
+                DSANLS_CUDA(cudaMemcpy2DAsync(h->M + r0 * h->ldM, h->ldM * sizeof(float), M + r0 * ld, ld * sizeof(float),
                                               h->n * sizeof(float), rc, cudaMemcpyHostToDevice, s));
                 DSANLS_CUDA(cudaEventRecord(h->ev_fork, s));
                 DSANLS_CUDA(cudaStreamWaitEvent(h->aux_stream, h->ev_fork, 0));
-                launch_transpose(h->M + r0 * h->n, h->n, rc, h->n, h->MT + r0, h->m, h->aux_stream);
+                launch_transpose(h->M + r0 * h->ldM, h->ldM, rc, h->n, h->MT + r0, h->ldT, h->aux_stream);
                 if (cast_b) launch_copy_cast_bf16(h->M + r0 * h->n, rc * h->n, h->Mb + r0 * h->n, h->aux_stream);
             }
             DSANLS_CUDA(cudaEventRecord(h->ev_join, h->aux_stream));
@@ -938,7 +1019,7 @@ int dsanls_set_dense(dsanls_t h, const float *M, int64_t ld, int32_t on_device) 
         // a graph holds the buffer pointers and, with the clamp, the bound by value
         if (!refresh || !had_copies || h->opt.bound_clamp) {
             invalidate_graph(h);
-            std::fill(h->cfg_key, h->cfg_key + 6, -1);
+            std::fill(h->cfg_key, h->cfg_key + 8, -1);
         }
         set_bound(h);
         DSANLS_CUDA(cudaStreamSynchronize(s));
@@ -1029,7 +1110,7 @@ int dsanls_set_csr(dsanls_t h, const int64_t *rowptr, const int32_t *col, const 
         launch_sumsq(h->cv, nnz, h->work, WORK_ELEMS, h->dscal + 0, s);
         h->has_sparse = true;
         invalidate_graph(h);
-        std::fill(h->cfg_key, h->cfg_key + 6, -1);
+        std::fill(h->cfg_key, h->cfg_key + 8, -1);
         set_bound(h);
         DSANLS_CUDA(cudaStreamSynchronize(s));  // host staging buffers go out of scope
         return DSANLS_OK;
@@ -1114,7 +1195,7 @@ int dsanls_rel_error(dsanls_t h, double *out) {
         factors_to_f32(h, s);
         if (h->has_dense) {
             ensure_sumsq(h);
-            launch_dense_residual(h->M, h->n, h->U, h->V, h->m, h->n, h->k, h->work, WORK_ELEMS, h->dscal + 1, s);
+            launch_dense_residual(h->M, h->ldM, h->U, h->V, h->m, h->n, h->k, h->work, WORK_ELEMS, h->dscal + 1, s);
         } else {
             double *GU = h->dscal + 3, *GV = h->dscal + 3 + 128 * 128;
             launch_sparse_cross(h->rp, h->ci, h->cv, h->m, h->U, h->V, h->k, h->work, WORK_ELEMS, h->dscal + 2, s);
@@ -1306,7 +1387,7 @@ void dsanls_destroy(dsanls_t h) {
         dfree(h->M); dfree(h->MT); dfree(h->Mb); dfree(h->MTb);
         dfree(h->rp); dfree(h->trp); dfree(h->ci); dfree(h->tci); dfree(h->cv); dfree(h->tcv);
         dfree(h->U); dfree(h->V); dfree(h->U16); dfree(h->V16);
-        dfree(h->S); dfree(h->Sb); dfree(h->J); dfree(h->A); dfree(h->W); dfree(h->Wpart); dfree(h->R);
+        dfree(h->S); dfree(h->Sb); dfree(h->J); dfree(h->A); dfree(h->W); dfree(h->Wpart); dfree(h->Gpart); dfree(h->Gparts); dfree(h->R);
         dfree(h->Rpart); dfree(h->Ytb); dfree(h->Bpart);
         dfree(h->P); dfree(h->Sn); dfree(h->Bb); dfree(h->Ptb); dfree(h->Ppart); dfree(h->Rpart2);
         dfree(h->Ptf); dfree(h->Pq); dfree(h->pscale); dfree(h->Spart);

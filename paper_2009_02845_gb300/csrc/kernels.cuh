@@ -89,6 +89,41 @@ void launch_sgemm(const GemmArgs &g, cudaStream_t s);
 void launch_split_reduce(const float *part, int64_t stride, int splits, int64_t M, int64_t N, int64_t ldp,
                          float *out, int64_t ldo, cudaStream_t s);
 
+// ---- gemm_split.cu --------------------------------------------------------
+// C[i][j] = alpha * sum_l a(i,l) b(j,l) at binary32 accuracy on tensor cores, from the
+// binary32 first operand (a(i,l) = A[i*lda + l] with a_kcontig, else
+// A[row(l)*lda + i], row(l) = gather[l] or l; any alignment) and the second one's
+// bf16 parts Bp[p][j][split_parts_ld(K)]: three of them (launch_split_parts), or one
+// when its values are bf16.  c_trans stores element (i, j) at C[j*ldc + i], else
+// at C[i*ldc + j].  `part` holds split_gemm_plan(M, N, K).part_elems floats; bit 2
+// of *err when a bounded wait gives up.
+struct SplitGemm {
+    int64_t M, N, K;
+    const float *A;
+    int64_t lda;
+    bool a_kcontig;
+    const int32_t *gather;
+    const __nv_bfloat16 *Bp;
+    int parts;
+    float *C;
+    int64_t ldc;
+    bool c_trans;
+    float alpha;
+    float *part;
+};
+struct SplitPlan {
+    int splits, kb_per_split;
+    int64_t part_elems;
+};
+SplitPlan split_gemm_plan(int64_t M, int64_t N, int64_t K);
+void launch_split_gemm(const SplitGemm &g, int *err, cudaStream_t s);
+int64_t split_parts_ld(int64_t K);
+// The three parts (3 N split_parts_ld(K) elements) of b(j,l) = B[j*ldb + l] with
+// kcontig, else B[row(l)*ldb + j].
+void launch_split_parts(const float *B, int64_t ldb, bool kcontig, const int32_t *gather, int64_t N, int64_t K,
+                        __nv_bfloat16 *out, cudaStream_t s);
+void prime_split_gemm_attributes(int max_smem);
+
 // ---- solver.cu ------------------------------------------------------------
 // Gram G = W W^T (W k x d, row-major fp32) accumulated in FP64; partials over
 // d-chunks reduced in fixed order.  Writes G64 (k x k).

@@ -499,6 +499,34 @@ void encode_bf16_map(CUtensorMap *out, const void *base, int64_t rows, int64_t c
     *out = make_map(base, rows, cols, box_rows);
 }
 
+namespace {
+CUtensorMap make_map_ld(CUtensorMapDataType type, int elem, CUtensorMapSwizzle swizzle, const void *base, int64_t rows,
+                        int64_t cols, int64_t ld, int box_cols, int box_rows) {
+    CUtensorMap m;
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)ld * elem};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = encode_fn()(&m, type, 2, const_cast<void *>(base), dims, strides, box, estr,
+                                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) throw ArgError{"cuTensorMapEncodeTiled failed"};
+    return m;
+}
+}  // namespace
+
+void encode_bf16_map_ld(CUtensorMap *out, const void *base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+    *out = make_map_ld(CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, CU_TENSOR_MAP_SWIZZLE_128B, base, rows, cols, ld, 64,
+                       box_rows);
+}
+
+void encode_f32_map(CUtensorMap *out, const void *base, int64_t rows, int64_t cols, int64_t ld, int box_cols,
+                    int box_rows, bool swizzle) {
+    *out = make_map_ld(CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4,
+                       swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, base, rows, cols, ld, box_cols,
+                       box_rows);
+}
+
 bool tc_supported(int k) { return k >= 1 && k <= 128; }
 
 int64_t tc_rpart_elems(int64_t rows, int64_t d, int k) {

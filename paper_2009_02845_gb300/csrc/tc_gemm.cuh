@@ -12,6 +12,12 @@ namespace dsanls {
 // base 16-byte aligned): boxes of 64 columns x box_rows rows, 128-byte swizzle
 // (the K-major operand layout of the tcgen05 kernels), zero fill out of bounds.
 void encode_bf16_map(CUtensorMap *out, const void *base, int64_t rows, int64_t cols, int box_rows);
+// the same with a row stride of ld >= cols elements (a multiple of 8)
+void encode_bf16_map_ld(CUtensorMap *out, const void *base, int64_t rows, int64_t cols, int64_t ld, int box_rows);
+// 2-D binary32 row-major tensor (row stride ld elements, a multiple of 4), box of box_cols x box_rows, with the
+// 128-byte swizzle (box_cols = 32) or none
+void encode_f32_map(CUtensorMap *out, const void *base, int64_t rows, int64_t cols, int64_t ld, int box_cols,
+                    int box_rows, bool swizzle);
 
 // True when the tcgen05 path handles rank k.
 bool tc_supported(int k);
