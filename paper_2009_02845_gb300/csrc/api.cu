@@ -285,7 +285,7 @@ SplitNeed split_need(const dsanls_ctx *h) {
         const int64_t rows = side == 0 ? h->m : h->n, K = side == 0 ? h->n : h->m, k = h->k;
         const int64_t dd = side == 0 ? h->d : d_v_of(h);
         auto use = [&](int64_t M, int64_t N, int64_t L) {
-            need.part = std::max(need.part, split_gemm_plan(M, N, L).part_elems);
+            need.part = std::max(need.part, split_gemm_plan(M, N, L, SPLIT_GEMM_MAX_SPLITS).part_elems);
             need.parts = std::max(need.parts, 3 * N * split_parts_ld(L));
         };
         if (h->sketch == DSANLS_SKETCH_SUBSAMPLE) {
@@ -452,7 +452,7 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
         }
         launch_split_parts(g.B, g.ldb, g.b_kcontig, g.gb, g.N, g.K, h->Gparts, s);
         launch_split_gemm(SplitGemm{g.M, g.N, g.K, g.A, g.lda, g.a_kcontig, g.ga, h->Gparts, 3, g.C, g.ldc, c_trans,
-                                    g.alpha, h->Gpart},
+                                    g.alpha, h->Gpart, SPLIT_GEMM_MAX_SPLITS},
                           h->flag, s);
     };
 

@@ -541,7 +541,7 @@ void launch_split_parts(const float *B, int64_t ldb, bool kcontig, const int32_t
     DSANLS_LAUNCH_CHECK();
 }
 
-SplitPlan split_gemm_plan(int64_t M, int64_t N, int64_t K) {
+SplitPlan split_gemm_plan(int64_t M, int64_t N, int64_t K, int max_splits) {
     const int bn = sg_bn(N);
     const int64_t tiles = ceil_div(M, SG_BM) * ceil_div(N, bn);
     const int nk = (int)ceil_div(K, SG_BK);
@@ -550,7 +550,7 @@ SplitPlan split_gemm_plan(int64_t M, int64_t N, int64_t K) {
     // read of their partial sums (8 bytes each at HBM rate), of which at most 256 MB are kept.
     int best = 1;
     double best_t = 1e30;
-    for (int sp = 1; sp <= std::min(nk, 64); ++sp) {
+    for (int sp = 1; sp <= std::min(nk, max_splits); ++sp) {
         const int kb = (int)ceil_div(nk, sp), real = (int)ceil_div(nk, kb);
         const double out = (double)sp * (double)M * (double)N;
         if (real != sp || (sp > 1 && out > 64.0e6)) continue;
@@ -574,7 +574,7 @@ void launch_split_gemm(const SplitGemm &g, int *err, cudaStream_t s) {
     if (g.gather && g.a_kcontig) throw ArgError{"split GEMM: a gather needs K rows"};
     if (g.M > (1ll << 31) - 1 || g.K > (1ll << 31) - 1 || 3 * g.N > (1ll << 31) - 1)
         throw ArgError{"sizes too large"};
-    const SplitPlan p = split_gemm_plan(g.M, g.N, g.K);
+    const SplitPlan p = split_gemm_plan(g.M, g.N, g.K, g.max_splits);
     float *dst = p.splits > 1 ? g.part : g.C;
     // partials keep C's orientation, so the reduction below is a plain sum of slices
     const int64_t rows = g.c_trans ? g.N : g.M, cols = g.c_trans ? g.M : g.N;

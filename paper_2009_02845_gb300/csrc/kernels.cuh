@@ -95,7 +95,8 @@ void launch_split_reduce(const float *part, int64_t stride, int splits, int64_t 
 // A[row(l)*lda + i], row(l) = gather[l] or l; any alignment) and the second one's
 // bf16 parts Bp[p][j][split_parts_ld(K)]: three of them (launch_split_parts), or one
 // when its values are bf16.  c_trans stores element (i, j) at C[j*ldc + i], else
-// at C[i*ldc + j].  `part` holds split_gemm_plan(M, N, K).part_elems floats; bit 2
+// at C[i*ldc + j].  `part` holds
+// split_gemm_plan(M, N, K, max_splits).part_elems floats; bit 2
 // of *err when a bounded wait gives up.
 struct SplitGemm {
     int64_t M, N, K;
@@ -110,12 +111,14 @@ struct SplitGemm {
     bool c_trans;
     float alpha;
     float *part;
+    int max_splits;
 };
 struct SplitPlan {
     int splits, kb_per_split;
     int64_t part_elems;
 };
-SplitPlan split_gemm_plan(int64_t M, int64_t N, int64_t K);
+SplitPlan split_gemm_plan(int64_t M, int64_t N, int64_t K, int max_splits);
+constexpr int SPLIT_GEMM_MAX_SPLITS = 64;
 void launch_split_gemm(const SplitGemm &g, int *err, cudaStream_t s);
 int64_t split_parts_ld(int64_t K);
 // The three parts (3 N split_parts_ld(K) elements) of b(j,l) = B[j*ldb + l] with

@@ -12,8 +12,15 @@
 //   Gn = (G + mu I) / s, s = tr(G + mu I) / k; bn = b / beta, beta = ||b|| / sqrt(k)
 // The weights used by the forward and backward passes are the fp32 master
 // weights rounded to bf16 (bf16 weights, fp32 accumulation); Adam updates the
-// fp32 masters.  All matrix products go through the CUDA-core GEMM of
-// gemm_simt.cu (deterministic); GELU is the exact x Phi(x) (normcdff).
+// fp32 masters.  Prediction's products run on tensor cores at binary32 accuracy
+// (gemm_split.cu: three-way bf16 splits; the weights are bf16 values, one part).
+// Training's stay binary32 chains in the order of the rows (gemm_simt.cu, k_colsum): Adam
+// divides by the gradient's own size and the weights are rounded to bf16 after every step,
+// so a rounding difference of 1e-7 in a gradient moves the weights by 1e-5 to 1e-4 within
+// 30 steps -- as far as the chain's own error, but a run would no longer repeat an earlier
+// one.  (Split products took 0.31 ms per step of 8,192 rows where these take 0.56; the
+// first form, one thread per column sum and 128 x 128 tiles, 6.5.)
+// Everything is deterministic; GELU is the exact x Phi(x) (normcdff).
 // Rows are grouped by subproblem: rows group_off[g] .. group_off[g+1]-1 share
 // G_g and mu_g.
 #include <algorithm>
@@ -32,11 +39,45 @@ namespace {
 DSANLS_DEV float gelu_f(float x) { return x * normcdff(x); }
 DSANLS_DEV float gelu_grad_f(float x) { return normcdff(x) + x * 0.3989422804014327f * __expf(-0.5f * x * x); }
 
-DSANLS_DEV float round_bf16(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+// A weight matrix (rows x cols at `off` of the parameters) as the second operand of
+// prediction's products: bf16 rows of split_parts_ld(cols).
+struct WeightParts {
+    int64_t off;
+    int rows, cols;
+    __nv_bfloat16 *n;
+};
 
-__global__ void k_round_bf16(const float *__restrict__ in, int64_t n, float *__restrict__ out) {
+DSANLS_DEV void put_parts(const WeightParts &w, int64_t i, __nv_bfloat16 q) {
+    const int64_t e = i - w.off;
+    if (e < 0 || e >= (int64_t)w.rows * w.cols) return;
+    const int64_t r = e / w.cols, c = e - r * w.cols;
+    w.n[r * ((w.cols + 7) / 8 * 8) + c] = q;
+}
+
+// wq = theta rounded to bf16, and the weights' operand copies.  With lr > 0 one Adam step
+// on theta first (the step and the rounding share one pass over the parameters).
+__global__ void k_adam_round(float *__restrict__ theta, float *__restrict__ m, float *__restrict__ v,
+                             const float *__restrict__ g, int64_t n, float lr, float b1, float b2, float c1, float c2,
+                             float eps, float *__restrict__ wq, WeightParts w0, WeightParts w1, WeightParts w2,
+                             WeightParts w3) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = round_bf16(in[i]);
+    if (i >= n) return;
+    float x = theta[i];
+    if (lr > 0.0f) {
+        const float gi = g[i];
+        const float mi = b1 * m[i] + (1.0f - b1) * gi;
+        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+        m[i] = mi;
+        v[i] = vi;
+        x -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        theta[i] = x;
+    }
+    const __nv_bfloat16 q = __float2bfloat16_rn(x);
+    wq[i] = __bfloat162float(q);
+    put_parts(w0, i, q);
+    put_parts(w1, i, q);
+    put_parts(w2, i, q);
+    put_parts(w3, i, q);
 }
 
 // per group: s_g and Gn_g
@@ -60,7 +101,7 @@ __global__ void k_norm_groups(const float *__restrict__ G, const float *__restri
     }
 }
 
-// per row: beta and bn; the row's group is found from group_off
+// the subproblem of row r, from group_off
 DSANLS_DEV int group_of(const int64_t *off, int ngroups, int64_t r) {
     int lo = 0, hi = ngroups;
     while (hi - lo > 1) {
@@ -73,102 +114,167 @@ DSANLS_DEV int group_of(const int64_t *off, int ngroups, int64_t r) {
     return lo;
 }
 
-__global__ void k_norm_rows(const float *__restrict__ b, int64_t rows, int k, float *__restrict__ bn,
-                            float *__restrict__ beta) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// one warp per row, one lane per column (k <= 32); the sum of squares in column order
+__global__ void __launch_bounds__(256) k_norm_rows(const float *__restrict__ b, int64_t rows, int k,
+                                                   float *__restrict__ bn, float *__restrict__ beta) {
+    const int lane = threadIdx.x & 31;
+    const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (r >= rows) return;
+    const float x = lane < k ? b[r * k + lane] : 0.0f;
     float ss = 0.0f;
-    for (int j = 0; j < k; ++j) ss = fmaf(b[r * k + j], b[r * k + j], ss);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        const float y = __shfl_sync(0xffffffffu, x, j);
+        ss = fmaf(y, y, ss);  // (zeros past k)
+    }
     float bt = sqrtf(ss / k);
     if (!(bt > 0.0f)) bt = 1.0f;
-    beta[r] = bt;
+    if (lane == 0) beta[r] = bt;
     const float inv = 1.0f / bt;
-    for (int j = 0; j < k; ++j) bn[r * k + j] = b[r * k + j] * inv;
+    if (lane < k) bn[r * k + lane] = x * inv;
 }
 
+// The activations: a CTA takes ACT_ROWS rows, threads the columns, so no element divides
+// for its row and column and a row's group is looked up once.
+constexpr int ACT_ROWS = 4;
+
 // z1 += zg[group] + b1 (in place), h1 = GELU(z1)
-__global__ void k_layer1_finish(float *__restrict__ z1, float *__restrict__ h1, const float *__restrict__ zg,
-                                const float *__restrict__ b1, const int64_t *__restrict__ off, int ngroups,
-                                int64_t rows, int h) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * h) return;
-    const int64_t r = idx / h;
-    const int j = (int)(idx % h);
-    const int g = group_of(off, ngroups, r);
-    const float z = z1[idx] + zg[(int64_t)g * h + j] + b1[j];
-    z1[idx] = z;
-    h1[idx] = gelu_f(z);
+__global__ void __launch_bounds__(256)
+    k_layer1_finish(float *__restrict__ z1, float *__restrict__ h1, const float *__restrict__ zg,
+                    const float *__restrict__ b1, const int64_t *__restrict__ off, int ngroups, int64_t rows, int h) {
+    __shared__ int grp[ACT_ROWS];
+    const int64_t r0 = (int64_t)blockIdx.x * ACT_ROWS;
+    if (threadIdx.x < ACT_ROWS) grp[threadIdx.x] = group_of(off, ngroups, min(rows - 1, r0 + threadIdx.x));
+    __syncthreads();
+    for (int j = threadIdx.x; j < h; j += blockDim.x) {
+        const float bj = b1[j];
+#pragma unroll
+        for (int i = 0; i < ACT_ROWS; ++i) {
+            if (r0 + i >= rows) break;
+            const int64_t idx = (r0 + i) * h + j;
+            const float z = z1[idx] + zg[(int64_t)grp[i] * h + j] + bj;
+            z1[idx] = z;
+            h1[idx] = gelu_f(z);
+        }
+    }
 }
 
 // z += bias (per column), act = GELU(z) or ReLU(z)
-__global__ void k_bias_act(float *__restrict__ z, float *__restrict__ act, const float *__restrict__ bias,
-                           int64_t rows, int cols, int relu) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * cols) return;
-    const float v = z[idx] + bias[idx % cols];
-    z[idx] = v;
-    act[idx] = relu ? fmaxf(v, 0.0f) : gelu_f(v);
+__global__ void __launch_bounds__(256)
+    k_bias_act(float *__restrict__ z, float *__restrict__ act, const float *__restrict__ bias, int64_t rows, int cols,
+               int relu) {
+    const int64_t r0 = (int64_t)blockIdx.x * ACT_ROWS * blockDim.y + threadIdx.y * ACT_ROWS;
+    for (int j = threadIdx.x; j < cols; j += blockDim.x) {
+        const float bj = bias[j];
+#pragma unroll
+        for (int i = 0; i < ACT_ROWS; ++i) {
+            if (r0 + i >= rows) break;
+            const int64_t idx = (r0 + i) * cols + j;
+            const float v = z[idx] + bj;
+            z[idx] = v;
+            act[idx] = relu ? fmaxf(v, 0.0f) : gelu_f(v);
+        }
+    }
 }
 
-// e = o - y* where y* > 0, max(o, 0) where y* = 0 (o before the ReLU);
-// do = e / N; per-row loss 1/2 ||e||^2.  Equal to the squared error of the
-// ReLU output except where o < 0 < y*, where it keeps a gradient.  ys and
-// dout may be the same array (each element is read before it is written).
-__global__ void k_out_grad(const float *__restrict__ o, const float *ys, int64_t rows, int k, float invN, float *dout,
-                           double *__restrict__ rowloss) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// The loss of a row against y* = x* s_g / beta_r: e = o - y* where y* > 0, max(o, 0)
+// where y* = 0 (o before the ReLU); do = e / N; 1/2 ||e||^2 to rowloss.  Equal to the squared
+// error of the ReLU output except where o < 0 < y*, where it keeps a gradient.  One warp
+// per row, one lane per column (k <= 32).
+__global__ void __launch_bounds__(256)
+    k_out_grad(const float *__restrict__ o, const float *__restrict__ xstar, const float *__restrict__ s_g,
+               const float *__restrict__ beta, const int64_t *__restrict__ off, int ngroups, int64_t rows, int k,
+               float invN, float *__restrict__ dout, double *__restrict__ rowloss) {
+    const int lane = threadIdx.x & 31;
+    const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (r >= rows) return;
     double l = 0.0;
-    for (int j = 0; j < k; ++j) {
-        const float oj = o[r * k + j], t = ys[r * k + j];
+    if (lane < k) {
+        const float oj = o[r * k + lane], t = xstar[r * k + lane] * s_g[group_of(off, ngroups, r)] / beta[r];
         const float e = t > 0.0f ? oj - t : fmaxf(oj, 0.0f);
-        l += 0.5 * (double)e * (double)e;
-        dout[r * k + j] = e * invN;
+        l = 0.5 * (double)e * (double)e;
+        dout[r * k + lane] = e * invN;
     }
-    rowloss[r] = l;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) l += __shfl_xor_sync(0xffffffffu, l, d);
+    if (lane == 0) rowloss[r] = l;
 }
 
-// dz = dh * GELU'(z)
-__global__ void k_gelu_back(const float *__restrict__ z, float *__restrict__ dh, int64_t n) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dh[i] *= gelu_grad_f(z[i]);
+// dh *= GELU'(z) in place (the backward pass through the activation)
+__global__ void __launch_bounds__(256) k_gelu_back(const float *__restrict__ z, float *__restrict__ dh, int64_t n) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        dh[i] *= gelu_grad_f(z[i]);
 }
 
-// out[g * cols + j] = sum over rows off[g] <= r < off[g+1] of X[r * cols + j] (row order)
-__global__ void k_segment_colsum(const float *__restrict__ X, const int64_t *__restrict__ off, int nseg, int cols,
-                                 float *__restrict__ out) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)nseg * cols) return;
-    const int g = (int)(idx / cols), j = (int)(idx % cols);
+// out[g * cols + j] = sum over rows off[g] <= r < off[g+1] of X[r * cols + j], one chain per
+// column in row order (off null: one segment of all rows).  A CTA takes 32 columns of a
+// segment: seven warps copy tiles of CS_ROWS rows ahead by cp.async, the first one adds.
+// Bound by the chain, four cycles per row (a thread that loaded each row itself took 1 ms
+// for 8,192 rows).
+constexpr int CS_ROWS = 112, CS_STAGES = 3;
+__global__ void __launch_bounds__(256) k_colsum(const float *__restrict__ X, const int64_t *__restrict__ off,
+                                                int64_t rows, int cols, float *__restrict__ out) {
+    __shared__ float tile[CS_STAGES][CS_ROWS][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, ctiles = (cols + 31) / 32;
+    const int64_t g = blockIdx.x / ctiles;
+    const int j = (int)(blockIdx.x % ctiles) * 32 + lane;
+    const int64_t r0 = off ? off[g] : 0, r1 = off ? off[g + 1] : rows;
+    const int64_t nt = r1 > r0 ? (r1 - r0 + CS_ROWS - 1) / CS_ROWS : 0;
+    auto fetch = [&](int64_t t) {
+        if (w == 0) return;
+#pragma unroll
+        for (int i = 0; i < CS_ROWS / 7; ++i) {
+            const int q = w - 1 + 7 * i;
+            const int64_t r = r0 + t * CS_ROWS + q;
+            const bool in = t < nt && r < r1 && j < cols;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(&tile[t % CS_STAGES][q][lane])),
+                         "l"(in ? X + r * cols + j : X), "r"(in ? 4 : 0)
+                         : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int t = 0; t < CS_STAGES - 1; ++t) fetch(t);
     float acc = 0.0f;
-    for (int64_t r = off[g]; r < off[g + 1]; ++r) acc += X[r * cols + j];
-    out[idx] = acc;
-}
-
-__global__ void k_sum_doubles(const double *__restrict__ x, int64_t n, double scale, double *__restrict__ out) {
-    __shared__ double red[256];
-    double v = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) v += x[i];
-    red[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
+    for (int64_t t = 0; t < nt; ++t) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(CS_STAGES - 2) : "memory");
+        __syncthreads();  // tile t has landed, tile t - 1 has been added
+        fetch(t + CS_STAGES - 1);
+        if (w == 0) {
+            const float(*x)[32] = tile[t % CS_STAGES];
+            const int n = (int)min((int64_t)CS_ROWS, r1 - r0 - t * CS_ROWS);
+            if (n == CS_ROWS) {
+#pragma unroll
+                for (int q = 0; q < CS_ROWS; q += 16) {
+                    float v[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) v[e] = x[q + e][lane];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) acc = __fadd_rn(acc, v[e]);
+                }
+            } else {
+                for (int r = 0; r < n; ++r) acc = __fadd_rn(acc, x[r][lane]);
+            }
+        }
     }
-    if (threadIdx.x == 0) *out = red[0] * scale;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (w == 0 && j < cols) out[g * cols + j] = acc;
 }
 
-__global__ void k_adam(float *__restrict__ theta, float *__restrict__ m, float *__restrict__ v,
-                       const float *__restrict__ g, int64_t n, float lr, float b1, float b2, float c1, float c2,
-                       float eps) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    theta[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+__global__ void __launch_bounds__(1024) k_sum_doubles(const double *__restrict__ x, int64_t n, double scale,
+                                                      double *__restrict__ out) {
+    __shared__ double red[32];
+    double v = 0.0;
+#pragma unroll 8
+    for (int64_t i = threadIdx.x; i < n; i += 1024) v += x[i];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        v = red[threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (threadIdx.x == 0) *out = v * scale;
+    }
 }
 
 __global__ void k_g_to_float(const double *__restrict__ G64, int k, const double *__restrict__ scal,
@@ -189,15 +295,25 @@ __global__ void k_rhs_b(const float *__restrict__ R, const float *__restrict__ Z
 
 unsigned nblk(int64_t n) { return (unsigned)ceil_div(n, 256); }
 
-GemmArgs gemm(int64_t M, int64_t N, int64_t K, const float *A, int64_t lda, bool ak, const float *B, int64_t ldb,
-              bool bk, float *C, int64_t ldc) {
-    GemmArgs g{};
-    g.M = M; g.N = N; g.K = K;
-    g.A = A; g.lda = lda; g.a_kcontig = ak;
-    g.B = B; g.ldb = ldb; g.b_kcontig = bk;
-    g.C = C; g.ldc = ldc; g.alpha = 1.0f; g.splits = 1;
-    return g;
+// C (M x N) = A W^T at binary32 accuracy on tensor cores, W's bf16 rows as parts (no split
+// of K: C holds as many rows as the batch)
+void times_weights(int64_t M, int64_t N, int64_t K, const float *A, const __nv_bfloat16 *W, float *C, int *err,
+                   cudaStream_t s) {
+    launch_split_gemm(SplitGemm{M, N, K, A, K, true, nullptr, W, 1, C, N, false, 1.0f, nullptr, 1}, err, s);
 }
+
+// one binary32 chain per output
+void chain(int64_t M, int64_t N, int64_t K, const float *A, int64_t lda, bool ak, const float *B, int64_t ldb, bool bk,
+           float *C, int64_t ldc, cudaStream_t s) {
+    launch_sgemm(GemmArgs{M, N, K, A, lda, nullptr, ak, B, ldb, nullptr, bk, C, ldc, 1.0f, 1, 0}, s);
+}
+
+void column_sums(const float *X, const int64_t *off, int nseg, int64_t rows, int cols, float *out, cudaStream_t s) {
+    k_colsum<<<(unsigned)(ceil_div(cols, 32) * nseg), 256, 0, s>>>(X, off, rows, cols, out);
+    DSANLS_LAUNCH_CHECK();
+}
+
+constexpr int MLP_MAX_SPLITS = 64;  // of the Gram layer's product
 
 }  // namespace
 
@@ -234,101 +350,156 @@ void mlp_alloc(MlpState &st, int k, int h, int64_t max_rows, int max_groups) {
     al(st.bn, max_rows * k); al(st.beta, max_rows);
     al(st.z1, max_rows * h); al(st.h1, max_rows * h); al(st.z2, max_rows * h); al(st.h2, max_rows * h);
     al(st.o, max_rows * k); al(st.y, max_rows * k); al(st.dout, max_rows * k); al(st.rowloss, max_rows);
-    al(st.loss, 1); al(st.all_off, 2);
+    al(st.loss, 2);  // the loss, then the error word
+    st.err = reinterpret_cast<int *>(st.loss + 1);
     al(st.gf1, (int64_t)k * k); al(st.mu1, 1); al(st.off1, 2);
+    al(st.W1g, h * split_parts_ld((int64_t)k * k)); al(st.W1b, h * split_parts_ld(k)); al(st.W2, h * split_parts_ld(h));
+    al(st.W3, k * split_parts_ld(h));
+    // split-K partials of the Gram layer (batches of few groups)
+    al(st.part, ceil_div((int64_t)k * k, 64) * std::min<int64_t>(max_groups, 19456) * h);
+    DSANLS_CUDA(cudaMemset(st.loss, 0, 2 * sizeof(double)));
     DSANLS_CUDA(cudaMemset(st.m, 0, P * sizeof(float)));
     DSANLS_CUDA(cudaMemset(st.v, 0, P * sizeof(float)));
-    const int64_t zero_n[2] = {0, 0};
-    DSANLS_CUDA(cudaMemcpy(st.all_off, zero_n, sizeof zero_n, cudaMemcpyHostToDevice));
+}
+
+void mlp_reserve_training(MlpState &st) {
+    if (!st.dz2 && cudaMalloc((void **)&st.dz2, (size_t)(st.max_rows * st.h) * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        st.dz2 = nullptr;
+        throw std::bad_alloc();
+    }
+    for (cudaStream_t &t : st.side)
+        if (!t) DSANLS_CUDA(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
+    for (cudaEvent_t *e : {&st.ev[0], &st.ev[1], &st.ev[2], &st.done[0], &st.done[1], &st.done[2]})
+        if (!*e) DSANLS_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
 }
 
 void mlp_free(MlpState &st) {
     for (void *p : {(void *)st.theta, (void *)st.wq, (void *)st.grad, (void *)st.m, (void *)st.v, (void *)st.Gn,
                     (void *)st.s, (void *)st.zg, (void *)st.dzg, (void *)st.bn, (void *)st.beta, (void *)st.z1,
                     (void *)st.h1, (void *)st.z2, (void *)st.h2, (void *)st.o, (void *)st.y, (void *)st.dout,
-                    (void *)st.rowloss, (void *)st.loss, (void *)st.all_off, (void *)st.gf1, (void *)st.mu1,
-                    (void *)st.off1})
+                    (void *)st.rowloss, (void *)st.loss, (void *)st.gf1, (void *)st.mu1, (void *)st.off1,
+                    (void *)st.W1g, (void *)st.W1b, (void *)st.W2, (void *)st.W3, (void *)st.part,
+                    (void *)st.dz2})
         if (p) cudaFree(p);
+    for (cudaStream_t t : st.side)
+        if (t) cudaStreamDestroy(t);
+    for (cudaEvent_t e : {st.ev[0], st.ev[1], st.ev[2], st.done[0], st.done[1], st.done[2]})
+        if (e) cudaEventDestroy(e);
     st = MlpState{};
 }
 
-void mlp_quantise(MlpState &st, cudaStream_t s) {
-    const int64_t P = mlp_param_count(st.k, st.h);
-    k_round_bf16<<<nblk(P), 256, 0, s>>>(st.theta, P, st.wq);
+// Adam step (lr > 0) and the rounded weights
+static void adam_round(MlpState &st, float lr, cudaStream_t s) {
+    const int k = st.k, h = st.h;
+    const MlpOffsets O = mlp_offsets(k, h);
+    float c1 = 1.0f, c2 = 1.0f;
+    const float b1 = 0.9f, b2 = 0.999f;
+    if (lr > 0.0f) {
+        st.adam_t += 1;
+        c1 = 1.0f - std::pow(b1, (float)st.adam_t);
+        c2 = 1.0f - std::pow(b2, (float)st.adam_t);
+    }
+    k_adam_round<<<nblk(O.total), 256, 0, s>>>(st.theta, st.m, st.v, st.grad, O.total, lr, b1, b2, c1, c2, 1e-8f, st.wq,
+                                               WeightParts{O.W1g, h, k * k, st.W1g},
+                                               WeightParts{O.W1b, h, k, st.W1b},
+                                               WeightParts{O.W2, h, h, st.W2},
+                                               WeightParts{O.W3, k, h, st.W3});
+    DSANLS_LAUNCH_CHECK();
+}
+
+void mlp_quantise(MlpState &st, cudaStream_t s) { adam_round(st, 0.0f, s); }
+void mlp_adam(MlpState &st, float lr, cudaStream_t s) { adam_round(st, lr, s); }
+
+static void bias_act(float *z, float *act, const float *bias, int64_t rows, int cols, int relu, cudaStream_t s) {
+    const unsigned tx = (unsigned)std::min(256, (cols + 31) / 32 * 32), ty = 256 / tx;
+    k_bias_act<<<(unsigned)ceil_div(rows, ACT_ROWS * ty), dim3(tx, ty), 0, s>>>(z, act, bias, rows, cols, relu);
     DSANLS_LAUNCH_CHECK();
 }
 
 // Forward pass: y (rows x k, normalised output) in st.y; o, z1, h1, z2, h2 kept.
 void mlp_forward(MlpState &st, const float *G, const float *mu, const int64_t *off, int ngroups, const float *b,
-                 int64_t rows, cudaStream_t s) {
+                 int64_t rows, bool training, int *err, cudaStream_t s) {
     const int k = st.k, h = st.h;
+    const int64_t kk = (int64_t)k * k;
     const MlpOffsets O = mlp_offsets(k, h);
     const float *W = st.wq;
     k_norm_groups<<<ngroups, 128, 0, s>>>(G, mu, k, ngroups, st.Gn, st.s);
     DSANLS_LAUNCH_CHECK();
-    launch_sgemm(gemm(ngroups, h, (int64_t)k * k, st.Gn, (int64_t)k * k, true, W + O.W1g, (int64_t)k * k, true, st.zg,
-                      h),
-                 s);
-    k_norm_rows<<<nblk(rows), 256, 0, s>>>(b, rows, k, st.bn, st.beta);
+    if (training)
+        chain(ngroups, h, kk, st.Gn, kk, true, W + O.W1g, kk, true, st.zg, h, s);
+    else
+        launch_split_gemm(SplitGemm{ngroups, h, kk, st.Gn, kk, true, nullptr, st.W1g, 1, st.zg, h, false, 1.0f, st.part,
+                                    ngroups <= 19456 ? MLP_MAX_SPLITS : 1},
+                          err, s);
+    k_norm_rows<<<(unsigned)ceil_div(rows, 8), 256, 0, s>>>(b, rows, k, st.bn, st.beta);
     DSANLS_LAUNCH_CHECK();
-    launch_sgemm(gemm(rows, h, k, st.bn, k, true, W + O.W1b, k, true, st.z1, h), s);
-    k_layer1_finish<<<nblk(rows * h), 256, 0, s>>>(st.z1, st.h1, st.zg, W + O.b1, off, ngroups, rows, h);
+    if (training)
+        chain(rows, h, k, st.bn, k, true, W + O.W1b, k, true, st.z1, h, s);
+    else
+        times_weights(rows, h, k, st.bn, st.W1b, st.z1, err, s);
+    k_layer1_finish<<<(unsigned)ceil_div(rows, ACT_ROWS), (unsigned)std::min(256, (h + 31) / 32 * 32), 0, s>>>(
+        st.z1, st.h1, st.zg, W + O.b1, off, ngroups, rows, h);
     DSANLS_LAUNCH_CHECK();
-    launch_sgemm(gemm(rows, h, h, st.h1, h, true, W + O.W2, h, true, st.z2, h), s);
-    k_bias_act<<<nblk(rows * h), 256, 0, s>>>(st.z2, st.h2, W + O.b2, rows, h, 0);
-    DSANLS_LAUNCH_CHECK();
-    launch_sgemm(gemm(rows, k, h, st.h2, h, true, W + O.W3, h, true, st.o, k), s);
-    k_bias_act<<<nblk(rows * k), 256, 0, s>>>(st.o, st.y, W + O.b3, rows, k, 1);
-    DSANLS_LAUNCH_CHECK();
+    if (training)
+        chain(rows, h, h, st.h1, h, true, W + O.W2, h, true, st.z2, h, s);
+    else
+        times_weights(rows, h, h, st.h1, st.W2, st.z2, err, s);
+    bias_act(st.z2, st.h2, W + O.b2, rows, h, 0, s);
+    if (training)
+        chain(rows, k, h, st.h2, h, true, W + O.W3, h, true, st.o, k, s);
+    else
+        times_weights(rows, k, h, st.h2, st.W3, st.o, err, s);
+    bias_act(st.o, st.y, W + O.b3, rows, k, 1, s);
 }
 
 // Loss and gradient (into st.grad) of the one-sided squared error (k_out_grad) after mlp_forward.
-void mlp_backward(MlpState &st, const int64_t *off, int ngroups, const float *ystar, int64_t rows, cudaStream_t s) {
+void mlp_backward(MlpState &st, const int64_t *off, int ngroups, const float *xstar, int64_t rows, cudaStream_t s) {
     const int k = st.k, h = st.h;
+    const int64_t kk = (int64_t)k * k;
     const MlpOffsets O = mlp_offsets(k, h);
     const float *W = st.wq;
     float *dG = st.grad;
-    k_out_grad<<<nblk(rows), 256, 0, s>>>(st.o, ystar, rows, k, 1.0f / (float)rows, st.dout, st.rowloss);
+    k_out_grad<<<(unsigned)ceil_div(rows, 8), 256, 0, s>>>(st.o, xstar, st.s, st.beta, off, ngroups, rows, k,
+                                                          1.0f / (float)rows, st.dout, st.rowloss);
     DSANLS_LAUNCH_CHECK();
-    k_sum_doubles<<<1, 256, 0, s>>>(st.rowloss, rows, 1.0 / (double)rows, st.loss);  // mean over rows
+    k_sum_doubles<<<1, 1024, 0, s>>>(st.rowloss, rows, 1.0 / (double)rows, st.loss);  // mean over rows
     DSANLS_LAUNCH_CHECK();
-    // dW3 = do^T h2, db3 = colsum(do)
-    launch_sgemm(gemm(k, h, rows, st.dout, k, false, st.h2, h, false, dG + O.W3, h), s);
-    const int64_t hostoff[2] = {0, rows};
-    DSANLS_CUDA(cudaMemcpyAsync(st.all_off, hostoff, sizeof hostoff, cudaMemcpyHostToDevice, s));
-    k_segment_colsum<<<nblk(k), 256, 0, s>>>(st.dout, st.all_off, 1, k, dG + O.b3);
+    const unsigned eb = (unsigned)std::min<int64_t>(ceil_div(rows * h, 256), 152 * 16);
+    // The weight gradients and the column sums are long chains on few SMs: they run beside the
+    // path to the lower layer on the side streams (0: dW3, 1: the column sums, 2: dW2), each
+    // from the event after its input, and join it at the end.  That path writes buffers whose
+    // last reader is behind it: dz2 has its own, dz1 takes z2's.
+    auto fork = [&](int e) { DSANLS_CUDA(cudaEventRecord(st.ev[e], s)); };
+    auto after = [&](int t, int e) { DSANLS_CUDA(cudaStreamWaitEvent(st.side[t], st.ev[e], 0)); };
+    fork(0);  // do
+    after(0, 0);
+    chain(k, h, rows, st.dout, k, false, st.h2, h, false, dG + O.W3, h, st.side[0]);  // dW3 = do^T h2
+    after(1, 0);
+    column_sums(st.dout, nullptr, 1, rows, k, dG + O.b3, st.side[1]);
+    chain(rows, h, k, st.dout, k, true, W + O.W3, h, false, st.dz2, h, s);  // dh2 = do W3 -> dz2
+    k_gelu_back<<<eb, 256, 0, s>>>(st.z2, st.dz2, rows * h);
     DSANLS_LAUNCH_CHECK();
-    // dh2 = do W3 -> dz2 (in h2's buffer)
-    launch_sgemm(gemm(rows, h, k, st.dout, k, true, W + O.W3, h, false, st.h2, h), s);
-    k_gelu_back<<<nblk(rows * h), 256, 0, s>>>(st.z2, st.h2, rows * h);
+    fork(1);  // dz2
+    after(2, 1);
+    chain(h, h, rows, st.dz2, h, false, st.h1, h, false, dG + O.W2, h, st.side[2]);  // dW2 = dz2^T h1
+    after(1, 1);
+    column_sums(st.dz2, nullptr, 1, rows, h, dG + O.b2, st.side[1]);
+    float *dz1 = st.z2;
+    chain(rows, h, h, st.dz2, h, true, W + O.W2, h, false, dz1, h, s);  // dh1 = dz2 W2 -> dz1
+    k_gelu_back<<<eb, 256, 0, s>>>(st.z1, dz1, rows * h);
     DSANLS_LAUNCH_CHECK();
-    // dW2 = dz2^T h1, db2
-    launch_sgemm(gemm(h, h, rows, st.h2, h, false, st.h1, h, false, dG + O.W2, h), s);
-    k_segment_colsum<<<nblk(h), 256, 0, s>>>(st.h2, st.all_off, 1, h, dG + O.b2);
-    DSANLS_LAUNCH_CHECK();
-    // dh1 = dz2 W2 -> dz1 (in h1's buffer)
-    launch_sgemm(gemm(rows, h, h, st.h2, h, true, W + O.W2, h, false, st.h1, h), s);
-    k_gelu_back<<<nblk(rows * h), 256, 0, s>>>(st.z1, st.h1, rows * h);
-    DSANLS_LAUNCH_CHECK();
-    // dW1b = dz1^T bn, db1, per-group dzg and dW1g = dzg^T Gn
-    launch_sgemm(gemm(h, k, rows, st.h1, h, false, st.bn, k, false, dG + O.W1b, k), s);
-    k_segment_colsum<<<nblk(h), 256, 0, s>>>(st.h1, st.all_off, 1, h, dG + O.b1);
-    DSANLS_LAUNCH_CHECK();
-    k_segment_colsum<<<nblk((int64_t)ngroups * h), 256, 0, s>>>(st.h1, off, ngroups, h, st.dzg);
-    DSANLS_LAUNCH_CHECK();
-    launch_sgemm(gemm(h, (int64_t)k * k, ngroups, st.dzg, h, false, st.Gn, (int64_t)k * k, false, dG + O.W1g,
-                      (int64_t)k * k),
-                 s);
-}
-
-void mlp_adam(MlpState &st, float lr, cudaStream_t s) {
-    const int64_t P = mlp_param_count(st.k, st.h);
-    st.adam_t += 1;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.0f - std::pow(b1, (float)st.adam_t), c2 = 1.0f - std::pow(b2, (float)st.adam_t);
-    k_adam<<<nblk(P), 256, 0, s>>>(st.theta, st.m, st.v, st.grad, P, lr, b1, b2, c1, c2, 1e-8f);
-    DSANLS_LAUNCH_CHECK();
-    mlp_quantise(st, s);
+    fork(2);  // dz1
+    after(1, 2);
+    column_sums(dz1, nullptr, 1, rows, h, dG + O.b1, st.side[1]);
+    // per-group dzg and dW1g = dzg^T Gn, dW1b = dz1^T bn
+    column_sums(dz1, off, ngroups, rows, h, st.dzg, s);
+    chain(h, kk, ngroups, st.dzg, h, false, st.Gn, kk, false, dG + O.W1g, kk, s);
+    chain(h, k, rows, dz1, h, false, st.bn, k, false, dG + O.W1b, k, s);
+    for (int t = 0; t < 3; ++t) {
+        DSANLS_CUDA(cudaEventRecord(st.done[t], st.side[t]));
+        DSANLS_CUDA(cudaStreamWaitEvent(s, st.done[t], 0));
+    }
 }
 
 __global__ void k_init_segment(float *__restrict__ theta, int64_t off, int64_t n, float a) {
@@ -355,26 +526,12 @@ void mlp_init(MlpState &st, uint64_t seed, cudaStream_t s) {
     mlp_quantise(st, s);
 }
 
-__global__ void k_targets(const float *__restrict__ xstar, const float *__restrict__ s_g,
-                          const float *__restrict__ beta, const int64_t *__restrict__ off, int ngroups, int64_t rows,
-                          int k, float *__restrict__ ys) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * k) return;
-    const int64_t r = idx / k;
-    ys[idx] = xstar[idx] * s_g[group_of(off, ngroups, r)] / beta[r];
-}
-
 __global__ void k_unscale(const float *__restrict__ y, const float *__restrict__ s_g, const float *__restrict__ beta,
                           const int64_t *__restrict__ off, int ngroups, int64_t rows, int k, float *__restrict__ x) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * k) return;
     const int64_t r = idx / k;
     x[idx] = y[idx] * beta[r] / s_g[group_of(off, ngroups, r)];
-}
-
-void mlp_targets(MlpState &st, const int64_t *off, int ngroups, const float *xstar, int64_t rows, cudaStream_t s) {
-    k_targets<<<nblk(rows * st.k), 256, 0, s>>>(xstar, st.s, st.beta, off, ngroups, rows, st.k, st.dout);
-    DSANLS_LAUNCH_CHECK();
 }
 
 void mlp_unscale(MlpState &st, const int64_t *off, int ngroups, int64_t rows, float *x_out, cudaStream_t s) {
@@ -467,7 +624,7 @@ void mlp_learned_update(MlpState &st, float *Z, const float *R, int64_t rows, co
     // b = R + mu Z into st.dout (rows x k) for the network input
     k_rhs_b<<<nblk(rows * k), 256, 0, s>>>(R, Z, scal, rows * k, st.dout);
     DSANLS_LAUNCH_CHECK();
-    mlp_forward(st, st.gf1, st.mu1, st.off1, 1, st.dout, rows, s);
+    mlp_forward(st, st.gf1, st.mu1, st.off1, 1, st.dout, rows, false, flag, s);
     const int64_t blocks = std::min<int64_t>(ceil_div(rows, LF_THREADS / 32), 152 * 8);
     k_learned_finish<<<(unsigned)blocks, LF_THREADS, 0, s>>>(Z, R, st.y, st.beta, st.s, Gf, kp, scal, rows, k,
                                                             pg_iters, plain_iters, kept, flag);

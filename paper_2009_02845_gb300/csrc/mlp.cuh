@@ -1,6 +1,7 @@
 // Learned warm start: network state and launchers (see mlp.cu).
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -23,7 +24,14 @@ struct MlpState {
     float *z1 = nullptr, *h1 = nullptr, *z2 = nullptr, *h2 = nullptr;
     float *o = nullptr, *y = nullptr, *dout = nullptr;
     double *rowloss = nullptr, *loss = nullptr;
-    int64_t *all_off = nullptr;
+    int *err = nullptr;  // raised when a product's bounded wait gives up (after the loss)
+    // the rounded weights as second operands of prediction's products
+    __nv_bfloat16 *W1g = nullptr, *W1b = nullptr, *W2 = nullptr, *W3 = nullptr;
+    float *part = nullptr;  // split-K partials
+    // training (from the first step on): dz2, and side streams with their events
+    float *dz2 = nullptr;
+    cudaStream_t side[3] = {nullptr, nullptr, nullptr};
+    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr}, done[3] = {nullptr, nullptr, nullptr};
     float *gf1 = nullptr, *mu1 = nullptr;  // single-group input of the learned update
     int64_t *off1 = nullptr;
 };
@@ -34,8 +42,11 @@ void mlp_alloc(MlpState &st, int k, int h, int64_t max_rows, int max_groups);
 void mlp_free(MlpState &st);
 void mlp_quantise(MlpState &st, cudaStream_t s);
 void mlp_forward(MlpState &st, const float *G, const float *mu, const int64_t *off, int ngroups, const float *b,
-                 int64_t rows, cudaStream_t s);
-void mlp_backward(MlpState &st, const int64_t *off, int ngroups, const float *ystar, int64_t rows, cudaStream_t s);
+                 int64_t rows, bool training, int *err, cudaStream_t s);
+// buffers and streams of the backward pass (at the first training step)
+void mlp_reserve_training(MlpState &st);
+// after a training forward pass: loss and gradient against y* = x* s_g / beta_r
+void mlp_backward(MlpState &st, const int64_t *off, int ngroups, const float *xstar, int64_t rows, cudaStream_t s);
 void mlp_adam(MlpState &st, float lr, cudaStream_t s);
 // Learned form of a half-step's update of Z (rows x k, k <= 32) from R, G (FP64 and
 // padded fp32 Gf with row stride kp) and scal = {lambda, mu, eta}; counts kept rows.
@@ -47,8 +58,6 @@ void mlp_harvest(const float *Z, const float *R, const float *Gf, int kp, const 
                  int iters, float *b_out, float *x_out, cudaStream_t s);
 // theta ~ U(-sqrt(3/fan_in), sqrt(3/fan_in)) from Philox stream 0x20 keyed by seed; biases 0.
 void mlp_init(MlpState &st, uint64_t seed, cudaStream_t s);
-// y* = x* s_g / beta_r (targets of the normalised problem) into st.dout after mlp_forward.
-void mlp_targets(MlpState &st, const int64_t *off, int ngroups, const float *xstar, int64_t rows, cudaStream_t s);
 // x0 = y beta_r / s_g (the warm start in the original scale) after mlp_forward.
 void mlp_unscale(MlpState &st, const int64_t *off, int ngroups, int64_t rows, float *x_out, cudaStream_t s);
 

@@ -2,6 +2,7 @@
 // prediction and one training step (forward, backward, Adam).
 #include <cuda_runtime.h>
 
+#include <cstring>
 #include <new>
 #include <string>
 
@@ -112,7 +113,7 @@ int dsanls_mlp_predict(dsanls_mlp_t m, const float *G, const float *mu, const in
     if (int rc = check_batch(m, G, mu, group_off, ngroups, b, rows)) return rc;
     return mguard([&]() {
         cudaStream_t s = (cudaStream_t)stream;
-        mlp_forward(m->st, G, mu, group_off, ngroups, b, rows, s);
+        mlp_forward(m->st, G, mu, group_off, ngroups, b, rows, false, m->st.err, s);
         mlp_unscale(m->st, group_off, ngroups, rows, x_out, s);
         return DSANLS_OK;
     });
@@ -129,15 +130,24 @@ int dsanls_mlp_train_step(dsanls_mlp_t m, const float *G, const float *mu, const
     }
     return mguard([&]() {
         cudaStream_t s = (cudaStream_t)stream;
-        mlp_forward(m->st, G, mu, group_off, ngroups, b, rows, s);
-        mlp_targets(m->st, group_off, ngroups, xstar, rows, s);
-        mlp_backward(m->st, group_off, ngroups, m->st.dout, rows, s);
+        mlp_reserve_training(m->st);
+        mlp_forward(m->st, G, mu, group_off, ngroups, b, rows, true, m->st.err, s);
+        mlp_backward(m->st, group_off, ngroups, xstar, rows, s);
         if (grad)
             DSANLS_CUDA(cudaMemcpyAsync(grad, m->st.grad, mlp_param_count(m->st.k, m->st.h) * sizeof(float),
                                         cudaMemcpyDeviceToHost, s));
-        if (loss) DSANLS_CUDA(cudaMemcpyAsync(loss, m->st.loss, sizeof(double), cudaMemcpyDeviceToHost, s));
+        double out[2] = {0.0, 0.0};  // the loss and the error word behind it
+        DSANLS_CUDA(cudaMemcpyAsync(out, m->st.loss, sizeof out, cudaMemcpyDeviceToHost, s));
         if (lr > 0.0f) mlp_adam(m->st, lr, s);
         DSANLS_CUDA(cudaStreamSynchronize(s));
+        if (loss) *loss = out[0];
+        int err = 0;
+        std::memcpy(&err, &out[1], sizeof err);
+        if (err) {
+            DSANLS_CUDA(cudaMemset(m->st.err, 0, sizeof(int)));
+            record_handleless_error("a bounded device wait gave up (tensor-core pipeline)");
+            return DSANLS_ETIMEOUT;
+        }
         return DSANLS_OK;
     });
 }
