@@ -166,6 +166,7 @@ struct dsanls_ctx {
     double *work = nullptr;
     int64_t *t_dev = nullptr;
     int *flag = nullptr;
+    __nv_bfloat16 *eparts = nullptr;  // split parts of U and V for the dense relative error
     double *dscal = nullptr;  // [0] ||M||^2, [1] residual^2, [2] cross, [3..] Gram of U, Gram of V
     uint32_t *bits = nullptr;  // membership bitmap of the sampled set (sparse subsampling)
     SubCsr sub[2];             // sub-CSR of X[:, J] per side (sparse data, subsampling sketch)
@@ -788,6 +789,7 @@ void prime_kernel_attributes() {
     prime_solver_attributes(max_smem);
     prime_tc_attributes(max_smem);
     prime_split_gemm_attributes(max_smem);
+    prime_residual_attributes(max_smem);
     batch_prime_tc(max_smem);
     done[dev] = true;
 }
@@ -1193,9 +1195,25 @@ int dsanls_rel_error(dsanls_t h, double *out) {
     return guarded(h, [&]() {
         cudaStream_t s = h->stream();
         factors_to_f32(h, s);
+        bool tc = false;
+        auto residual = [&]() {
+            launch_dense_residual(h->M, h->ldM, h->U, h->V, h->m, h->n, h->k, h->work, WORK_ELEMS, h->dscal + 1, s);
+        };
         if (h->has_dense) {
             ensure_sumsq(h);
-            launch_dense_residual(h->M, h->ldM, h->U, h->V, h->m, h->n, h->k, h->work, WORK_ELEMS, h->dscal + 1, s);
+            tc = residual_tc_supported(h->ldM, h->m, h->n, h->k);
+            if (tc && !h->eparts) {
+                try {
+                    dalloc(h->eparts, residual_tc_parts(h->m, h->n, h->k));
+                } catch (const std::bad_alloc &) {
+                    tc = false;  // no room for the parts: the form that needs none
+                }
+            }
+            if (tc)
+                launch_dense_residual_tc(h->M, h->ldM, h->U, h->V, h->m, h->n, h->k, h->dscal + 0, h->eparts, h->work,
+                                         WORK_ELEMS, h->dscal + 1, h->flag, s);
+            else
+                residual();
         } else {
             double *GU = h->dscal + 3, *GV = h->dscal + 3 + 128 * 128;
             launch_sparse_cross(h->rp, h->ci, h->cv, h->m, h->U, h->V, h->k, h->work, WORK_ELEMS, h->dscal + 2, s);
@@ -1206,6 +1224,11 @@ int dsanls_rel_error(dsanls_t h, double *out) {
         if (int rc = pending_status(h)) return rc;
         double v[2];
         DSANLS_CUDA(cudaMemcpy(v, h->dscal, 2 * sizeof(double), cudaMemcpyDeviceToHost));
+        if (tc && !std::isfinite(v[1])) {  // residuals out of binary32's range against M: squares in FP64
+            residual();
+            if (int rc = pending_status(h)) return rc;
+            DSANLS_CUDA(cudaMemcpy(v, h->dscal, 2 * sizeof(double), cudaMemcpyDeviceToHost));
+        }
         *out = v[0] > 0.0 ? std::sqrt(std::max(v[1], 0.0) / v[0]) : 0.0;
         return DSANLS_OK;
     });
@@ -1400,7 +1423,7 @@ void dsanls_destroy(dsanls_t h) {
             dfree(h->scal[side]);
         }
         dfree(h->Gf); dfree(h->work); dfree(h->t_dev); dfree(h->flag); dfree(h->dscal);
-        dfree(h->bits); dfree(h->kept);
+        dfree(h->bits); dfree(h->kept); dfree(h->eparts);
         h->sub[0].release();
         h->sub[1].release();
         if (h->aux_stream) {

@@ -468,15 +468,14 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
 }
 
 // Parts of a second operand: out[p][n][ldk], ldk = K rounded up to 8.
-// K contiguous in B (row n at B + n ldb): one thread per element.
+// K contiguous in B (row n at B + n ldb): blockDim.x along K, blockDim.y and the grid along the rows.
 __global__ void k_parts_rows(const float *__restrict__ B, int64_t ldb, int64_t N, int64_t K, int64_t ldk,
                              __nv_bfloat16 *__restrict__ out) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    for (int64_t n = blockIdx.y; n < N; n += gridDim.y) {
-        __nv_bfloat16 *o = out + n * ldk + k;
-        split3_one(B[n * ldb + k], o[0], o[N * ldk], o[2 * N * ldk]);
-    }
+    for (int64_t n = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; n < N; n += (int64_t)gridDim.x * blockDim.y)
+        for (int64_t k = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; k < K; k += (int64_t)gridDim.y * blockDim.x) {
+            __nv_bfloat16 *o = out + n * ldk + k;
+            split3_one(B[n * ldb + k], o[0], o[N * ldk], o[2 * N * ldk]);
+        }
 }
 
 // N contiguous in B (element (n, k) at B[row(k) ldb + n], row(k) = gather[k] or k)
@@ -531,8 +530,10 @@ void launch_split_parts(const float *B, int64_t ldb, bool kcontig, const int32_t
     if (N <= 0 || K <= 0) return;
     const int64_t ldk = split_parts_ld(K);
     if (kcontig) {
-        k_parts_rows<<<dim3((unsigned)ceil_div(K, 256), (unsigned)std::min<int64_t>(N, 65535)), 256, 0, s>>>(
-            B, ldb, N, K, ldk, out);
+        const int tx = K <= 32 ? 32 : (K <= 64 ? 64 : (K <= 128 ? 128 : 256)), ty = 256 / tx;
+        const dim3 grid((unsigned)std::min<int64_t>(ceil_div(N, ty), 152 * 16),
+                        (unsigned)std::min<int64_t>(ceil_div(K, tx), 64));
+        k_parts_rows<<<grid, dim3(tx, ty), 0, s>>>(B, ldb, N, K, ldk, out);
     } else {
         if (ceil_div(N, 32) > 65535) throw ArgError{"split parts: too many rows"};
         k_parts_cols<<<dim3((unsigned)ceil_div(K, 32), (unsigned)ceil_div(N, 32)), dim3(32, 8), 0, s>>>(
