@@ -391,8 +391,8 @@ void prepare(dsanls_ctx *h) {
     if (h->sketch == DSANLS_SKETCH_SUBSAMPLE && h->has_sparse) {
         // U-half: columns of M (rows of M^T), V-half: rows of M; room for the
         // longest possible sampled set of each side
-        h->sub[0].reserve(m, h->d, top_sum(h->h_trp, h->d), h->stream());
-        h->sub[1].reserve(n, dv, top_sum(h->h_rp, dv), h->stream());
+        h->sub[0].reserve(m, h->d, top_sum(h->h_trp, h->d), (double)h->nnz * h->d / ((double)m * n), h->stream());
+        h->sub[1].reserve(n, dv, top_sum(h->h_rp, dv), (double)h->nnz * dv / ((double)m * n), h->stream());
     } else {
         h->sub[0].release();
         h->sub[1].release();
@@ -789,6 +789,7 @@ void prime_kernel_attributes() {
     prime_solver_attributes(max_smem);
     prime_tc_attributes(max_smem);
     prime_split_gemm_attributes(max_smem);
+    prime_update_attributes(max_smem);
     prime_residual_attributes(max_smem);
     batch_prime_tc(max_smem);
     done[dev] = true;

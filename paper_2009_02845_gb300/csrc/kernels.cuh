@@ -201,15 +201,24 @@ void launch_spmm_rows(const int64_t *rowptr, const int32_t *col, const float *va
 // Rows of a sub-CSR with more than this many entries are long: their right-hand
 // side is summed by a whole CTA (launch_subcsr_rows, launch_subcsr_long_rows).
 constexpr int64_t SUB_LONG = 64;
+// Rows of more than this many are left to a warp each where one thread would walk them.
+constexpr int64_t SUB_MID = 16;
+// The entries are placed row by row and the rows sorted (instead of a radix sort over all
+// entries) when a row is expected to hold at most this many.
+constexpr double SUB_PLACE_AVG = 8.0;
 
 struct SubCsr {
     int64_t rows = 0, cap = 0;
     int dmax = 0, cur = 0;
     int64_t *off = nullptr, *len = nullptr, *bsum = nullptr, *hist = nullptr, *ptr = nullptr;
-    int32_t *cnt = nullptr, *longs = nullptr;  // longs: count, then the rows with many entries
+    int32_t *cnt = nullptr, *longs = nullptr;  // longs: count, then the rows of more than SUB_LONG entries
+    int32_t *mids = nullptr;  // count, then the rows of SUB_MID + 1 .. SUB_LONG entries; null: not listed
+    bool place = false;       // rows placed and sorted (else radix-sorted entries)
     int32_t *key[2] = {nullptr, nullptr}, *col[2] = {nullptr, nullptr};
     float *val[2] = {nullptr, nullptr};
-    void reserve(int64_t rows, int dmax, int64_t cap, cudaStream_t s);
+    // per_row: the entries a row is expected to hold
+    void reserve(int64_t rows, int dmax, int64_t cap, double per_row, cudaStream_t s);
+    int64_t warp_rows() const { return mids ? SUB_MID : SUB_LONG; }  // longer rows: launch_subcsr_long_rows
     void release();
 };
 // Build the sub-CSR of X[:, J] from the CSR of X^T (xtp, xtc, xtv); J ascending, d <= dmax.
@@ -220,7 +229,7 @@ void launch_subcsr_build(const int64_t *xtp, const int32_t *xtc, const float *xt
 // rows by a CTA (32 interleaved partial sums added in a fixed order).
 template <typename T>
 void launch_subcsr_rows(const SubCsr &sc, const T *Y, int64_t yrows, int k, float alpha, float *out, cudaStream_t s);
-// only the long rows (more than SUB_LONG entries) of launch_subcsr_rows
+// only the rows of more than sc.warp_rows() entries of launch_subcsr_rows, with its sums
 template <typename T>
 void launch_subcsr_long_rows(const SubCsr &sc, const T *Y, int64_t yrows, int k, float alpha, float *out,
                              cudaStream_t s);

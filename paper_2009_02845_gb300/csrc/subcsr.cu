@@ -9,15 +9,26 @@
 //   2. gather: entry e of the concatenation (p-major, so in ascending column
 //      order) goes to position e with key = its row of X, col = J_p, val;
 //      cnt[row] += 1;
-//   3. stable LSD radix sort of (key, col, val) by key, 8 bits per pass, so
-//      every row's entries stay in ascending column order -- the CSR order of
-//      the row in X, which makes sums over a row deterministic and equal to a
-//      row-wise pass over X that skips the unsampled columns;
-//   4. ptr = exclusive scan of cnt (rows + 1), and cnt cleared for the next build.
+//   3. the entries by row, in ascending e within a row: the CSR order of the row in X,
+//      which makes sums over a row deterministic and equal to a row-wise pass over X that
+//      skips the unsampled columns.  In one of two ways, by the expected number of sampled
+//      entries per row (SubCsr::reserve):
+//      few (<= SUB_PLACE_AVG): ptr = exclusive scan of cnt; every entry's e to the next free
+//      place of its row, in whatever order the atomics fall; then each row is sorted by e --
+//      a row of <= SUB_MID entries by one thread, <= SUB_LONG by a warp, longer ones by a
+//      CTA's radix sort -- and its columns and values are fetched.  9 launches that each
+//      touch an entry or a row once: what bounds them is the random access (a 4-byte
+//      atomic, a 4-byte store and two 4-byte loads per entry), not bytes;
+//      many: stable LSD radix sort of (key, col, val) by key, 8 bits per pass (5 launches a
+//      pass, 19 in all for 2e6 rows), whose cost does not grow with the length of a row;
+//      ptr = exclusive scan of cnt, and cnt cleared for the next build.
+//   2e6 x 5e5 with 1.4e6 / 3.6e5 sampled entries (0.7 per row on both sides, up to 4,800 in
+//   one of V's), build and long rows' sums: radix 302 / 230 us, placed 153 / 191 (gather 27,
+//   place 22, sort 48 of the first; sort of the long rows 40 and their sums 35 of the
+//   second).  The line SUB_PLACE_AVG: a thread of k_sort_rows reads n^2 places for a row of
+//   n, which at 8 is still what the radix passes move; SUB_MID bounds the longest.
 // Every size that changes with J lives in device memory, so the build is
 // captured once in the iteration's CUDA graph; the launch grids are fixed.
-// Reads ~12 bytes per sampled entry per pass and 16 bytes per row, instead
-// of the 4 bytes per stored entry of X of a bitmap scan over every row.
 #include <algorithm>
 #include <new>
 
@@ -121,6 +132,34 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(const In *__restrict
 
 // ---- gather of the sampled columns ----------------------------------------------
 // len[p] = length of row J[p] of X^T
+// One CTA does it with the scan when d is small: off[0..d], the launches saved.
+constexpr int SEG_SCAN_MAX = 1 << 16;
+__global__ void __launch_bounds__(SCAN_THREADS) k_seg_scan(const int64_t *__restrict__ xtp, const int32_t *__restrict__ J,
+                                                           int d, int64_t *__restrict__ off) {
+    __shared__ int64_t wt[SCAN_THREADS / 32];
+    constexpr int PER = SCAN_CHUNK / SCAN_THREADS;
+    int64_t base = 0;
+    for (int b0 = 0; b0 < d; b0 += SCAN_CHUNK) {
+        const int i0 = b0 + threadIdx.x * PER;
+        int64_t v[PER], loc = 0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            v[j] = i0 + j < d ? xtp[J[i0 + j] + 1] - xtp[J[i0 + j]] : 0;
+            loc += v[j];
+        }
+        int64_t total;
+        int64_t run = base + block_excl_scan(loc, wt, &total);
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            if (i0 + j < d) off[i0 + j] = run;
+            run += v[j];
+        }
+        base += total;
+        __syncthreads();  // wt is free again
+    }
+    if (threadIdx.x == 0) off[d] = base;
+}
+
 __global__ void k_seg_len(const int64_t *__restrict__ xtp, const int32_t *__restrict__ J, int d,
                           int64_t *__restrict__ len) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -144,7 +183,11 @@ __global__ void __launch_bounds__(256)
         const int32_t j = __ldg(&J[lo]);
         const int64_t src = __ldg(&xtp[j]) + (e - __ldg(&off[lo]));
         const int32_t row = xtc[src];
-        if (!DSANLS_IN(e, cap, 101) || !DSANLS_IN(row, rows, 102)) continue;
+        if (!DSANLS_IN(e, cap, 101)) continue;
+        if (!DSANLS_IN(row, rows, 102)) {
+            key[e] = -1;
+            continue;
+        }
         key[e] = row;
         col[e] = j;
         val[e] = xtv[src];
@@ -221,15 +264,153 @@ __global__ void __launch_bounds__(RADIX_THREADS)
     }
 }
 
+// ---- placement and sort of short rows ------------------------------------------------
+// place[ptr[row] + ...] = e for every entry; cnt is 0 again afterwards.
+__global__ void __launch_bounds__(256)
+    k_place(const int32_t *__restrict__ key, const int64_t *__restrict__ total_p, const int64_t *__restrict__ ptr,
+            int32_t *__restrict__ cnt, int32_t *__restrict__ place) {
+    const int64_t total = *total_p;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t row = key[e];
+        if (row < 0) continue;
+        const int64_t at = ptr[row] + atomicSub(&cnt[row], 1) - 1;
+        if (DSANLS_IN(at, total, 106)) place[at] = (int32_t)e;
+    }
+}
+
+// Rows of at most SUB_MID entries, one thread each: an entry's place is the number of
+// smaller e of its row.  Longer rows are listed.
+__global__ void __launch_bounds__(256)
+    k_sort_rows(const int64_t *__restrict__ ptr, int64_t rows, const int32_t *__restrict__ place,
+                const int32_t *__restrict__ col, const float *__restrict__ val, int32_t *__restrict__ ocol,
+                float *__restrict__ oval, int32_t *__restrict__ longs, int32_t *__restrict__ mids) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e0 = ptr[i];
+        const int64_t n64 = ptr[i + 1] - e0;
+        if (n64 > SUB_LONG) {
+            longs[1 + atomicAdd(longs, 1)] = (int32_t)i;
+        } else if (n64 > SUB_MID) {
+            mids[1 + atomicAdd(mids, 1)] = (int32_t)i;
+        } else {
+            const int n = (int)n64;
+            for (int a = 0; a < n; ++a) {
+                const int32_t e = place[e0 + a];
+                int r = 0;
+                for (int b = 0; b < n; ++b) r += place[e0 + b] < e;
+                ocol[e0 + r] = col[e];
+                oval[e0 + r] = val[e];
+            }
+        }
+    }
+}
+
+// The listed rows: a warp per row of at most SUB_LONG entries (two per lane), and a CTA per
+// longer row, LSD radix by 8 bits of e between `place` and `tmp` (the row's own range of
+// both), as many passes as the total has digits.
+constexpr int LIST_THREADS = 1024;
+__global__ void __launch_bounds__(LIST_THREADS)
+    k_sort_listed(const int64_t *__restrict__ ptr, const int64_t *__restrict__ total_p, int32_t *__restrict__ place,
+                  int32_t *__restrict__ tmp, const int32_t *__restrict__ col, const float *__restrict__ val,
+                  int32_t *__restrict__ ocol, float *__restrict__ oval, const int32_t *__restrict__ longs,
+                  const int32_t *__restrict__ mids) {
+    __shared__ int base[256];
+    __shared__ int wcnt[LIST_THREADS / 32][256];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t total = *total_p;
+    const int nlong = longs[0], nmid = mids[0];
+    for (int l = blockIdx.x; l < nlong; l += gridDim.x) {
+        const int64_t e0 = ptr[longs[1 + l]];
+        const int n = (int)(ptr[longs[1 + l] + 1] - e0);
+        int32_t *a = place + e0, *b = tmp + e0;
+        for (int shift = 0; shift < 32 && (total >> shift) > 0; shift += 8) {
+            if (tid < 256) base[tid] = 0;
+            __syncthreads();
+            for (int i = tid; i < n; i += LIST_THREADS) atomicAdd(&base[(a[i] >> shift) & 255], 1);
+            __syncthreads();
+            if (warp == 0) {  // exclusive scan of the 256 counts
+                int run = 0;
+                for (int c = lane; c < 256; c += 32) {
+                    const int v = base[c];
+                    int x = v;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, x, o);
+                        if (lane >= o) x += y;
+                    }
+                    base[c] = run + x - v;
+                    run += __shfl_sync(0xffffffffu, x, 31);
+                }
+            }
+            for (int t0 = 0; t0 < n; t0 += LIST_THREADS) {
+                for (int c = tid; c < LIST_THREADS / 32 * 256; c += LIST_THREADS) (&wcnt[0][0])[c] = 0;
+                __syncthreads();
+                const bool ok = t0 + tid < n;
+                const int32_t e = ok ? a[t0 + tid] : 0;
+                const int dig = ok ? (e >> shift) & 255 : 256;
+                const unsigned peers = __match_any_sync(0xffffffffu, dig);
+                const int lrank = __popc(peers & ((1u << lane) - 1u));
+                if (ok && lrank == 0) wcnt[warp][dig] = __popc(peers);
+                __syncthreads();
+                if (tid < 256) {  // counts -> first positions, warp by warp
+                    int run = base[tid];
+                    for (int w = 0; w < LIST_THREADS / 32; ++w) {
+                        const int v = wcnt[w][tid];
+                        wcnt[w][tid] = run;
+                        run += v;
+                    }
+                    base[tid] = run;
+                }
+                __syncthreads();
+                if (ok) {
+                    const int at = wcnt[warp][dig] + lrank;
+                    if (DSANLS_IN(at, n, 107)) b[at] = e;
+                }
+                __syncthreads();
+            }
+            int32_t *const c = a;
+            a = b;
+            b = c;
+        }
+        for (int i = tid; i < n; i += LIST_THREADS) {
+            ocol[e0 + i] = col[a[i]];
+            oval[e0 + i] = val[a[i]];
+        }
+        __syncthreads();
+    }
+    for (int64_t l = (int64_t)blockIdx.x * (LIST_THREADS / 32) + warp; l < nmid;
+         l += (int64_t)gridDim.x * (LIST_THREADS / 32)) {
+        const int64_t e0 = ptr[mids[1 + l]];
+        const int n = (int)(ptr[mids[1 + l] + 1] - e0);
+        const int32_t x = lane < n ? place[e0 + lane] : 0, y = 32 + lane < n ? place[e0 + 32 + lane] : 0;
+        int rx = 0, ry = 0;
+        for (int i = 0; i < n; ++i) {
+            const int32_t v = i < 32 ? __shfl_sync(0xffffffffu, x, i) : __shfl_sync(0xffffffffu, y, i - 32);
+            rx += v < x;
+            ry += v < y;
+        }
+        if (lane < n) {
+            ocol[e0 + rx] = col[x];
+            oval[e0 + rx] = val[x];
+        }
+        if (32 + lane < n) {
+            ocol[e0 + ry] = col[y];
+            oval[e0 + ry] = val[y];
+        }
+    }
+}
+
 // ---- the right-hand side from the sub-CSR ----------------------------------------
 // Rows with more than SUB_LONG sampled entries (popular columns of a skewed
-// matrix gather thousands) are listed by k_long_rows and summed by a whole CTA
+// matrix gather thousands) are listed and summed by a whole CTA
 // of 32 warps; the rest by one warp each.
 
-__global__ void k_long_rows(const int64_t *__restrict__ ptr, int64_t rows, int32_t *__restrict__ list,
-                            int32_t *__restrict__ nlong) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows; i += (int64_t)gridDim.x * blockDim.x)
-        if (ptr[i + 1] - ptr[i] > SUB_LONG) list[atomicAdd(nlong, 1)] = (int32_t)i;
+__global__ void k_long_rows(const int64_t *__restrict__ ptr, int64_t rows, int32_t *__restrict__ longs,
+                            int32_t *__restrict__ mids) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t n = ptr[i + 1] - ptr[i];
+        if (n > SUB_LONG) longs[1 + atomicAdd(longs, 1)] = (int32_t)i;
+        else if (mids && n > SUB_MID) mids[1 + atomicAdd(mids, 1)] = (int32_t)i;
+    }
 }
 
 // out[i][c] = alpha * sum over the row's entries (ascending column) of val * Y[col][c]
@@ -265,17 +446,43 @@ __global__ void __launch_bounds__(256)
 // One CTA of LONG_WARPS warps per long row: warp w sums the entries e0 + w,
 // e0 + w + LONG_WARPS, ... (lanes across the k columns, four entries' loads in
 // flight), then the partial sums are added in warp order.
-constexpr int LONG_WARPS = 32;
+constexpr int LONG_WARPS = 32, LONG_CTAS = 304;
 
 template <typename T>
 __global__ void __launch_bounds__(32 * LONG_WARPS)
     k_sub_rows_long(const int64_t *__restrict__ ptr, const int32_t *__restrict__ col, const float *__restrict__ val,
                     const int32_t *__restrict__ list, const int32_t *__restrict__ nlong, const T *__restrict__ Y,
-                    int64_t yrows, int k, float alpha, float *__restrict__ out) {
+                    int64_t yrows, int k, float alpha, float *__restrict__ out, const int32_t *__restrict__ mids) {
     __shared__ float part[LONG_WARPS][128];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (blockIdx.x >= LONG_CTAS) {  // rows of more than SUB_MID entries: the sums of k_sub_rows
+        const int nm = mids[0];
+        for (int64_t l = (int64_t)(blockIdx.x - LONG_CTAS) * LONG_WARPS + warp; l < nm;
+             l += (int64_t)(gridDim.x - LONG_CTAS) * LONG_WARPS) {
+            const int64_t i = mids[1 + l];
+            const int64_t e1 = ptr[i + 1];
+            float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+            for (int64_t e = ptr[i]; e < e1; ++e) {
+                const float v = val[e];
+                if (!DSANLS_IN(col[e], yrows, 108)) continue;
+                const T *y = Y + (int64_t)col[e] * k;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int c = lane + 32 * q;
+                    if (c < k) acc[q] = __fmaf_rn(v, load_as_float(y + c), acc[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int c = lane + 32 * q;
+                if (c < k) out[i * k + c] = __fmul_rn(alpha, acc[q]);
+            }
+        }
+        return;
+    }
     const int n = *nlong;
-    for (int l = blockIdx.x; l < n; l += gridDim.x) {
+    for (int l = blockIdx.x; l < n; l += LONG_CTAS) {
         const int64_t i = list[l];
         const int64_t e0 = ptr[i], e1 = ptr[i + 1];
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -326,6 +533,7 @@ int key_passes(int64_t rows) {
 
 void SubCsr::release() {
     cudaFree(off); cudaFree(len); cudaFree(bsum); cudaFree(hist); cudaFree(ptr); cudaFree(cnt); cudaFree(longs);
+    cudaFree(mids);
     for (int b = 0; b < 2; ++b) {
         cudaFree(key[b]);
         cudaFree(col[b]);
@@ -342,9 +550,13 @@ static void sub_alloc(void **p, size_t bytes) {
     }
 }
 
-void SubCsr::reserve(int64_t rows_, int dmax_, int64_t cap_, cudaStream_t s) {
+void SubCsr::reserve(int64_t rows_, int dmax_, int64_t cap_, double per_row, cudaStream_t s) {
     if (rows_ > (1ll << 31) - 1) throw ArgError{"sub-CSR: more than 2^31 - 1 rows"};
-    if (rows == rows_ && dmax >= dmax_ && cap >= cap_ && off) return;
+    const bool few = per_row <= SUB_PLACE_AVG;
+    if (rows == rows_ && dmax >= dmax_ && cap >= cap_ && off) {
+        place = few && mids && cap < (1ll << 31);
+        return;
+    }
     release();
     rows = rows_;
     dmax = dmax_;
@@ -363,19 +575,48 @@ void SubCsr::reserve(int64_t rows_, int dmax_, int64_t cap_, cudaStream_t s) {
         sub_alloc((void **)&col[b], sizeof(int32_t) * (size_t)cap);
         sub_alloc((void **)&val[b], sizeof(float) * (size_t)cap);
     }
+    // the list of the rows of more than SUB_MID entries likewise; without room for it the
+    // radix sort and the longer rows' own sums serve
+    if (cudaMalloc((void **)&mids, sizeof(int32_t) * ((size_t)std::min<int64_t>(rows, cap / SUB_MID + 1) + 1)) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        mids = nullptr;
+    }
+    place = few && mids && cap < (1ll << 31);
     DSANLS_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)rows, s));
 }
 
 void launch_subcsr_build(const int64_t *xtp, const int32_t *xtc, const float *xtv, const int32_t *J, int d,
                          SubCsr &sc, cudaStream_t s) {
     if (d < 1 || d > sc.dmax) throw ArgError{"sub-CSR: sketch size outside the reserved range"};
-    k_seg_len<<<(unsigned)ceil_div(d, 256), 256, 0, s>>>(xtp, J, d, sc.len);
-    DSANLS_LAUNCH_CHECK();
-    launch_scan<int64_t>(sc.len, d, sc.bsum, sc.off, s);
+    if (d <= SEG_SCAN_MAX) {
+        k_seg_scan<<<1, SCAN_THREADS, 0, s>>>(xtp, J, d, sc.off);
+        DSANLS_LAUNCH_CHECK();
+    } else {
+        k_seg_len<<<(unsigned)ceil_div(d, 256), 256, 0, s>>>(xtp, J, d, sc.len);
+        DSANLS_LAUNCH_CHECK();
+        launch_scan<int64_t>(sc.len, d, sc.bsum, sc.off, s);
+    }
     k_gather<<<152 * 8, 256, 0, s>>>(xtp, xtc, xtv, J, sc.off, d, sc.key[0], sc.col[0], sc.val[0], sc.cnt, sc.cap,
                                      sc.rows);
     DSANLS_LAUNCH_CHECK();
     const int64_t *total = sc.off + d;
+    const unsigned row_ctas = (unsigned)std::min<int64_t>(ceil_div(sc.rows, 256), 152 * 8);
+    DSANLS_CUDA(cudaMemsetAsync(sc.longs, 0, sizeof(int32_t), s));
+    if (sc.mids) DSANLS_CUDA(cudaMemsetAsync(sc.mids, 0, sizeof(int32_t), s));
+    if (sc.place) {
+        launch_scan<int32_t>(sc.cnt, sc.rows, sc.bsum, sc.ptr, s);
+        k_place<<<152 * 8, 256, 0, s>>>(sc.key[0], total, sc.ptr, sc.cnt, sc.key[1]);
+        DSANLS_LAUNCH_CHECK();
+        k_sort_rows<<<row_ctas, 256, 0, s>>>(sc.ptr, sc.rows, sc.key[1], sc.col[0], sc.val[0], sc.col[1], sc.val[1],
+                                             sc.longs, sc.mids);
+        DSANLS_LAUNCH_CHECK();
+        k_sort_listed<<<304, LIST_THREADS, 0, s>>>(sc.ptr, total, sc.key[1], sc.key[0], sc.col[0], sc.val[0],
+                                                   sc.col[1], sc.val[1], sc.longs, sc.mids);
+        DSANLS_LAUNCH_CHECK();
+        sc.cur = 1;
+        return;
+    }
     const int passes = key_passes(sc.rows);
     for (int ps = 0; ps < passes; ++ps) {
         const int a = ps & 1;
@@ -390,9 +631,7 @@ void launch_subcsr_build(const int64_t *xtp, const int32_t *xtc, const float *xt
     sc.cur = passes & 1;
     launch_scan<int32_t>(sc.cnt, sc.rows, sc.bsum, sc.ptr, s);
     DSANLS_CUDA(cudaMemsetAsync(sc.cnt, 0, sizeof(int32_t) * (size_t)sc.rows, s));
-    DSANLS_CUDA(cudaMemsetAsync(sc.longs, 0, sizeof(int32_t), s));
-    k_long_rows<<<(unsigned)std::min<int64_t>(ceil_div(sc.rows, 256), 152 * 8), 256, 0, s>>>(sc.ptr, sc.rows,
-                                                                                           sc.longs + 1, sc.longs);
+    k_long_rows<<<row_ctas, 256, 0, s>>>(sc.ptr, sc.rows, sc.longs, sc.mids);
     DSANLS_LAUNCH_CHECK();
 }
 
@@ -404,8 +643,8 @@ void launch_subcsr_rows(const SubCsr &sc, const T *Y, int64_t yrows, int k, floa
     k_sub_rows<T><<<(unsigned)blocks, 256, 0, s>>>(sc.ptr, sc.col[sc.cur], sc.val[sc.cur], sc.rows, Y, yrows, k, alpha,
                                                    out);
     DSANLS_LAUNCH_CHECK();
-    k_sub_rows_long<T><<<152 * 2, 32 * LONG_WARPS, 0, s>>>(sc.ptr, sc.col[sc.cur], sc.val[sc.cur], sc.longs + 1,
-                                                           sc.longs, Y, yrows, k, alpha, out);
+    k_sub_rows_long<T><<<LONG_CTAS, 32 * LONG_WARPS, 0, s>>>(sc.ptr, sc.col[sc.cur], sc.val[sc.cur], sc.longs + 1,
+                                                           sc.longs, Y, yrows, k, alpha, out, nullptr);
     DSANLS_LAUNCH_CHECK();
 }
 template void launch_subcsr_rows<float>(const SubCsr &, const float *, int64_t, int, float, float *, cudaStream_t);
@@ -416,8 +655,8 @@ template <typename T>
 void launch_subcsr_long_rows(const SubCsr &sc, const T *Y, int64_t yrows, int k, float alpha, float *out,
                              cudaStream_t s) {
     if (sc.rows <= 0) return;
-    k_sub_rows_long<T><<<152 * 2, 32 * LONG_WARPS, 0, s>>>(sc.ptr, sc.col[sc.cur], sc.val[sc.cur], sc.longs + 1,
-                                                           sc.longs, Y, yrows, k, alpha, out);
+    k_sub_rows_long<T><<<LONG_CTAS + (sc.mids ? 152 : 0), 32 * LONG_WARPS, 0, s>>>(sc.ptr, sc.col[sc.cur], sc.val[sc.cur], sc.longs + 1,
+                                                           sc.longs, Y, yrows, k, alpha, out, sc.mids);
     DSANLS_LAUNCH_CHECK();
 }
 template void launch_subcsr_long_rows<float>(const SubCsr &, const float *, int64_t, int, float, float *,

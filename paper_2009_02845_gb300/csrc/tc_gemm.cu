@@ -29,7 +29,6 @@
 #include <algorithm>
 #include <mutex>
 
-#include "bounds.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
 #include "tc_gemm.cuh"
@@ -943,452 +942,12 @@ void launch_tc_skinny_split3(const __nv_bfloat16 *const X3[3], const __nv_bfloat
     launch_split_reduce(part, rows * k, p.splits, rows, k, k, R, k, s);
 }
 
-// ---- fused row update on tensor cores ---------------------------------------
-// Z <- max(0, Z - eta (Z G - R)) (eq. gradient_descent, one projected-gradient
-// step) for 32 < k <= 128.  Z G is taken on tcgen05 from a three-way bf16 split
-// of both operands, z = z_h + z_m + z_l with z_h = bf16(z), z_m = bf16(z - z_h),
-// z_l = bf16(z - z_h - z_m) (each difference exact in binary32): the six
-// products z_i g_j with i + j <= 2 accumulate in fp32 in TMEM, and the dropped
-// terms are of order 2^-24 |z| |g|, the rounding level of a binary32 product.
-//
-// Persistent, one CTA per SM.  The CTA splits G once into the three B operands
-// in shared memory (N = k rounded up to 16 rows, K = k rounded up to 64,
-// 128-byte swizzled K-major), then walks 128-row tiles of Z.  A tile of Z is
-// nr x k contiguous elements; it arrives in shared memory by one bulk copy,
-// issued two tiles ahead into a double buffer, so the reads of Z are in flight
-// while earlier tiles are computed.  Thread (row, slice) owns one row of the
-// tile and 32 consecutive columns: it reads its z from the buffer, writes the
-// split parts straight into tensor memory as the A operand (row i in lane i),
-// starts its loads of r, and after the MMAs (issued by one thread) reads its 32
-// accumulator columns back, applies the step and stores the row slice of Z.
-// Nothing of the tile passes through shared memory but the z read once.
-namespace {
-
-constexpr int UPD_BM = 128;
-
-struct __align__(8) UpdTail {
-    uint64_t full[2];  // the Z tile in buffer 0 / 1 has landed (bulk copy bytes)
-    uint64_t done;     // the tile's MMAs have retired
-    uint64_t fin;
-    uint32_t tmem_base;
-    uint32_t pad;
-};
-
-DSANLS_DEV float upd_project(float v, float bound, int *flag) {
-    if (!(fabsf(v) <= 3.402823466e38f)) {  // NaN or Inf
-        *flag = 1;
-        return 0.0f;
-    }
-    float r = v > 0.0f ? v : 0.0f;
-    if (bound > 0.0f) r = fminf(r, bound);
-    return r;
-}
-
-DSANLS_DEV uint32_t bf16_bits(__nv_bfloat16 v) { return (uint32_t)__bfloat16_as_ushort(v); }
-
-// Z of type ZT: binary32, or bf16 for the bf16-factor form -- z is then exactly
-// a bf16 value (z_m = z_l = 0), so only the three products z_h g_j are issued,
-// and the step's binary32 result is rounded to bf16 when it is stored.
-// The 32 elements of a row slice, `n` of them valid (the rest read as 0), from
-// shared or global memory; vectorised when the row start is 16 / 8 bytes aligned.
-DSANLS_DEV void load_slice(const float *p, int n, bool vec, float (&z)[32]) {
-    if (vec) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (4 * j < n) v = *reinterpret_cast<const float4 *>(p + 4 * j);
-            z[4 * j] = v.x, z[4 * j + 1] = v.y, z[4 * j + 2] = v.z, z[4 * j + 3] = v.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) z[j] = j < n ? p[j] : 0.0f;
-    }
-}
-DSANLS_DEV void load_slice(const __nv_bfloat16 *p, int n, bool vec, float (&z)[32]) {
-    if (vec) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            uint2 u = make_uint2(0u, 0u);
-            if (4 * j < n) u = *reinterpret_cast<const uint2 *>(p + 4 * j);
-            z[4 * j] = __uint_as_float(u.x << 16), z[4 * j + 1] = __uint_as_float(u.x & 0xffff0000u);
-            z[4 * j + 2] = __uint_as_float(u.y << 16), z[4 * j + 3] = __uint_as_float(u.y & 0xffff0000u);
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) z[j] = j < n ? __bfloat162float(p[j]) : 0.0f;
-    }
-}
-// Four consecutive elements, `n` of them valid (vectorised as load_slice).
-DSANLS_DEV void load4(const float *p, int n, bool vec, float (&y)[4]) {
-    if (vec) {
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (n >= 4) v = *reinterpret_cast<const float4 *>(p);
-        y[0] = v.x, y[1] = v.y, y[2] = v.z, y[3] = v.w;
-    } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) y[u] = u < n ? p[u] : 0.0f;
-    }
-}
-DSANLS_DEV void load4(const __nv_bfloat16 *p, int n, bool vec, float (&y)[4]) {
-    if (vec) {
-        uint2 w = make_uint2(0u, 0u);
-        if (n >= 4) w = *reinterpret_cast<const uint2 *>(p);
-        y[0] = __uint_as_float(w.x << 16), y[1] = __uint_as_float(w.x & 0xffff0000u);
-        y[2] = __uint_as_float(w.y << 16), y[3] = __uint_as_float(w.y & 0xffff0000u);
-    } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) y[u] = u < n ? __bfloat162float(p[u]) : 0.0f;
-    }
-}
-DSANLS_DEV void store4(float *p, float a, float b, float c, float d) {
-    *reinterpret_cast<float4 *>(p) = make_float4(a, b, c, d);
-}
-DSANLS_DEV void store4(__nv_bfloat16 *p, float a, float b, float c, float d) {
-    *reinterpret_cast<uint2 *>(p) = make_uint2(pack_bf16(a, b), pack_bf16(c, d));
-}
-
-template <int KA>  // K atoms of 64 columns: 1 for k <= 64, 2 for k <= 128
-__host__ __device__ constexpr int upd_threads() {
-    return KA * 256;  // 128 rows x (64 KA / 32) column slices
-}
-
-// Sparse subsampled data (SPR): the right-hand side of a row of at most SUB_LONG
-// sub-CSR entries is formed in the kernel, r = alpha * sum over the row's entries
-// (ascending) of val * Y[col][.], one fused multiply-add per entry and column --
-// the arithmetic of launch_subcsr_rows bit for bit -- so R is neither written nor
-// read for it; longer rows come precomputed in R (launch_subcsr_long_rows).
-template <typename ZT>
-struct UpdSub {
-    const int64_t *ptr;
-    const int32_t *col;
-    const float *val;
-    const ZT *Y;
-    int64_t yrows;
-    float alpha;
-};
-
-template <int KA, typename ZT, bool SPR>
-__global__ void __launch_bounds__(upd_threads<KA>())
-    k_update_tc(ZT *__restrict__ Z, const float *__restrict__ R, int64_t rows, int k, int N,
-                const float *__restrict__ Gf, int kp, const double *__restrict__ scal, float bound,
-                int *__restrict__ flag, uint32_t tmem_cols, int zbuf_bytes, int use_bulk, UpdSub<ZT> sub) {
-    constexpr bool ZBF = sizeof(ZT) == 2;
-    constexpr int ZPARTS = ZBF ? 1 : 3;  // nonzero parts of the split of z
-    constexpr int THREADS = upd_threads<KA>();
-    constexpr int KC = KA * 64;          // padded K
-    constexpr int ACOL = KA * 64;        // TMEM: accumulator in columns [0, N), the A parts from ACOL
-    extern __shared__ uint8_t upd_smem_raw[];
-    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(upd_smem_raw) + 1023) & ~uintptr_t(1023));
-    const int b_part = KA * N * 128;
-    uint8_t *Bp = base;  // 3 parts x KA atoms x N rows x 128 B
-    ZT *zbuf[2] = {reinterpret_cast<ZT *>(Bp + 3 * b_part), reinterpret_cast<ZT *>(Bp + 3 * b_part + zbuf_bytes)};
-    UpdTail *tail = reinterpret_cast<UpdTail *>(Bp + 3 * b_part + 2 * zbuf_bytes);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q = warp & 3, cw = warp >> 2;  // TMEM lane quarter and 32-column slice of this warp
-    const int row = 32 * q + lane, c0 = 32 * cw;
-    const int ncol = min(32, k - c0);  // valid columns of the slice (<= 0: padding only)
-    const bool vec = (k & 3) == 0;
-    const size_t es = sizeof(ZT);
-    if (tid == 0) {
-        mbar_init(&tail->full[0], 1);
-        mbar_init(&tail->full[1], 1);
-        mbar_init(&tail->done, 1);
-        mbar_init(&tail->fin, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(&tail->tmem_base)),
-                     "r"(tmem_cols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    // the three parts of G: B row n, K column c holds G[n][c] (G is symmetric)
-    for (int e = tid; e < N * KC; e += THREADS) {
-        const int n = e / KC, c = e % KC;
-        const float g = (n < k && c < k) ? Gf[n * kp + c] : 0.0f;
-        __nv_bfloat16 h, m, l;
-        split3_one(g, h, m, l);
-        const int off = sw128_off(n, c, N);
-        *reinterpret_cast<__nv_bfloat16 *>(Bp + off) = h;
-        *reinterpret_cast<__nv_bfloat16 *>(Bp + b_part + off) = m;
-        *reinterpret_cast<__nv_bfloat16 *>(Bp + 2 * b_part + off) = l;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    fence_before();
-    __syncthreads();
-    fence_after();
-    const uint32_t tmem = tail->tmem_base;
-    const uint32_t tlane = (uint32_t)(32 * q) << 16;
-    const float eta = (float)scal[2];
-    const uint32_t idesc = idesc_bf16(UPD_BM, N);
-    const int KS = (k + 15) >> 4;  // K steps of 16 that hold data
-    const int64_t ntiles = (rows + UPD_BM - 1) / UPD_BM;
-    // tile j of this CTA and whether it comes by bulk copy (every tile but a
-    // ragged last one whose byte count is not a multiple of 16)
-    auto tile_of = [&](int64_t j) { return (int64_t)blockIdx.x + j * gridDim.x; };
-    auto nrows = [&](int64_t t) { return (int)min((int64_t)UPD_BM, rows - t * UPD_BM); };
-    auto by_bulk = [&](int64_t t) { return use_bulk && (((int64_t)nrows(t) * k * (int64_t)es) & 15) == 0; };
-    uint32_t armed = 0;  // thread 0: buffers with a copy in flight
-    auto issue = [&](int64_t j) {
-        const int64_t t = tile_of(j);
-        if (t >= ntiles || !by_bulk(t)) return;
-        const int b = (int)(j & 1);
-        const uint32_t bytes = (uint32_t)((int64_t)nrows(t) * k * (int64_t)es);
-        mbar_expect_tx(&tail->full[b], bytes);
-        bulk_load(zbuf[b], Z + t * UPD_BM * (int64_t)k, bytes, &tail->full[b]);
-        armed |= 1u << b;
-    };
-    if (tid == 0) {
-        issue(0);
-        issue(1);
-    }
-    uint32_t phase = 0;  // bit b: parity of the next completion of full[b]
-    for (int64_t j = 0;; ++j) {
-        const int64_t tile = tile_of(j);
-        if (tile >= ntiles) break;
-        const int b = (int)(j & 1);
-        const int nr = nrows(tile);
-        const int64_t f0 = tile * UPD_BM * (int64_t)k;
-        const bool rowok = row < nr;
-        const int nv = rowok ? ncol : 0;  // valid entries of this thread's slice
-        // 1. r of the row slice: in flight while z is split and the products run
-        //    (SPR: the row's entry range now, r while the products run)
-        float rv[32];
-        int64_t e0 = 0, e1 = 0;
-        if (!SPR) {
-            load_slice(R + f0 + (int64_t)row * k + c0, nv, vec, rv);
-        } else if (rowok) {
-            e0 = sub.ptr[tile * UPD_BM + row];
-            e1 = sub.ptr[tile * UPD_BM + row + 1];
-        }
-        // 2. z of the row slice, from the bulk-copied buffer (or from Z for a ragged
-        //    last tile); the split parts go to tensor memory as the A operand
-        bool ok = true;
-        const bool bulk = by_bulk(tile);
-        if (bulk) {
-            ok = mbar_wait(&tail->full[b], (phase >> b) & 1, wait_limit());
-            if (ok) {
-                phase ^= 1u << b;
-                if (tid == 0) armed &= ~(1u << b);
-            }
-        }
-        float zv[32];
-        if (ok) {
-            const ZT *src = bulk ? zbuf[b] + row * k + c0 : Z + f0 + (int64_t)row * k + c0;
-            load_slice(src, nv, vec, zv);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) zv[e] = 0.0f;
-        }
-        if (ZBF) {  // z is a bf16 value: its split is z itself
-            uint32_t pk[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e)
-                pk[e] = (__float_as_uint(zv[2 * e]) >> 16) | (__float_as_uint(zv[2 * e + 1]) & 0xffff0000u);
-            tmem_st16(tmem + tlane + ACOL + cw * 16, pk);
-        } else {
-            uint32_t ph[16], pm[16], pl[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                __nv_bfloat16 h0, m0, l0, h1, m1, l1;
-                split3_one(zv[2 * e], h0, m0, l0);
-                split3_one(zv[2 * e + 1], h1, m1, l1);
-                ph[e] = bf16_bits(h0) | (bf16_bits(h1) << 16);
-                pm[e] = bf16_bits(m0) | (bf16_bits(m1) << 16);
-                pl[e] = bf16_bits(l0) | (bf16_bits(l1) << 16);
-            }
-            tmem_st16(tmem + tlane + ACOL + cw * 16, ph);
-            tmem_st16(tmem + tlane + ACOL + (KC / 2) + cw * 16, pm);
-            tmem_st16(tmem + tlane + ACOL + KC + cw * 16, pl);
-        }
-        tmem_st_wait();
-        fence_before();
-        if (__syncthreads_or(!ok)) {  // A complete in TMEM; the buffer b is read
-            if (tid == 0) atomicOr(flag, 2);
-            break;
-        }
-        fence_after();
-        // 3. the products into TMEM; the freed buffer takes tile j + 2
-        if (tid == 0) {
-            issue(j + 2);
-            const uint32_t b0 = smem_u32(Bp);
-            uint32_t acc = 0;
-#pragma unroll 1
-            for (int i = 0; i < ZPARTS; ++i)
-#pragma unroll 1
-                for (int jp = 0; i + jp < 3; ++jp)
-#pragma unroll 1
-                    for (int ks = 0; ks < KS; ++ks) {
-                        const uint32_t bd = b0 + jp * b_part + (ks >> 2) * N * 128 + (ks & 3) * 32;
-                        mma_bf16_tmem_a(tmem, tmem + ACOL + i * (KC / 2) + ks * 8, sw128_desc(bd), idesc, acc);
-                        acc = 1;
-                    }
-            mma_commit(&tail->done);
-        }
-        if (SPR) {
-            if (e1 - e0 > SUB_LONG) {
-                load_slice(R + f0 + (int64_t)row * k + c0, nv, vec, rv);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 32; ++c) rv[c] = 0.0f;
-                for (int64_t e = e0; e < e1; ++e) {
-                    const float v = sub.val[e];
-                    const int32_t yr = sub.col[e];
-                    if (!DSANLS_IN(yr, sub.yrows, 301)) continue;
-                    const ZT *y = sub.Y + (int64_t)yr * k + c0;
-#pragma unroll
-                    for (int q4 = 0; q4 < 8; ++q4) {
-                        float y4[4];
-                        load4(y + 4 * q4, nv - 4 * q4, vec, y4);
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) rv[4 * q4 + u] = __fmaf_rn(v, y4[u], rv[4 * q4 + u]);
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < 32; ++c) rv[c] = __fmul_rn(sub.alpha, rv[c]);
-            }
-        }
-        const bool got = mbar_wait(&tail->done, (uint32_t)(j & 1), wait_limit());
-        if (__syncthreads_or(!got)) {
-            if (tid == 0) atomicOr(flag, 2);
-            break;
-        }
-        fence_after();
-        // 4. the step on the row slice: Z G from the accumulator columns c0.., z
-        //    exact in registers, r loaded at the start of the tile
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            uint32_t a[16];
-            tmem_ld16(tmem + tlane + c0 + 16 * hh, a);
-            tmem_ld_wait();
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int c = 16 * hh + e;
-                const float grad = __fsub_rn(__uint_as_float(a[e]), rv[c]);
-                zv[c] = upd_project(__fmaf_rn(-eta, grad, zv[c]), bound, flag);
-            }
-        }
-        ZT *dst = Z + f0 + (int64_t)row * k + c0;
-        if (vec) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (4 * e < nv) store4(dst + 4 * e, zv[4 * e], zv[4 * e + 1], zv[4 * e + 2], zv[4 * e + 3]);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 32; ++e)
-                if (e < nv) dst[e] = store_cast<ZT>(zv[e]);
-        }
-        // the next tile's tcgen05.st and MMAs come after every thread's loads of
-        // the accumulator (the barrier after the next split orders them)
-        fence_before();
-    }
-    if (tid == 0) {  // every MMA and copy this thread issued has completed before TMEM and the CTA go
-        mma_commit(&tail->fin);
-        mbar_wait(&tail->fin, 0, wait_limit());
-        for (int b = 0; b < 2; ++b)
-            if (armed & (1u << b)) mbar_wait(&tail->full[b], (phase >> b) & 1, wait_limit());
-    }
-    fence_before();
-    __syncthreads();
-    fence_after();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
-}
-
-int update_tc_zbuf_bytes(int k, size_t es) { return (int)((UPD_BM * (size_t)k * es + 127) / 128 * 128); }
-
-template <int KA>
-size_t update_tc_smem(int N, int zbuf_bytes) {
-    return 1024 + 3 * (size_t)KA * N * 128 + 2 * (size_t)zbuf_bytes + sizeof(UpdTail);
-}
-
-}  // namespace
-
-bool update_tc_supported(int k) { return k > 32 && k <= 128; }
-
-namespace {
-template <int KA, typename ZT, bool SPR>
-void launch_update_tc_kind(ZT *Z, const float *R, int64_t rows, int k, int N, const float *Gf, int kp,
-                           const double *scal, float bound, int *flag, int sms, UpdSub<ZT> sub, cudaStream_t s) {
-    constexpr int zparts = sizeof(ZT) == 2 ? 1 : 3;
-    const int need = KA * 64 + zparts * KA * 32;  // accumulator + A parts, TMEM columns
-    uint32_t tmem_cols = 32;
-    while ((int)tmem_cols < need) tmem_cols <<= 1;
-    const int zb = update_tc_zbuf_bytes(k, sizeof(ZT));
-    const size_t smem = update_tc_smem<KA>(N, zb);
-    const int use_bulk = (reinterpret_cast<uintptr_t>(Z) & 15) == 0;
-    const int64_t ntiles = (rows + UPD_BM - 1) / UPD_BM;
-    const int64_t grid = std::min<int64_t>(ntiles, sms);  // one CTA per SM (shared memory and TMEM)
-    k_update_tc<KA, ZT, SPR><<<(unsigned)grid, upd_threads<KA>(), smem, s>>>(Z, R, rows, k, N, Gf, kp, scal, bound,
-                                                                             flag, tmem_cols, zb, use_bulk, sub);
-    DSANLS_LAUNCH_CHECK();
-}
-
-template <typename ZT, bool SPR>
-void launch_update_tc_any(ZT *Z, const float *R, int64_t rows, int k, const float *Gf, int kp, const double *scal,
-                          float bound, int *flag, UpdSub<ZT> sub, cudaStream_t s) {
-    if (!update_tc_supported(k)) throw ArgError{"launch_update_tc: needs 32 < k <= 128"};
-    if (rows <= 0) return;
-    const int N = (k + 15) / 16 * 16;
-    int dev = 0, sms = 152;
-    DSANLS_CUDA(cudaGetDevice(&dev));
-    DSANLS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (k <= 64)
-        launch_update_tc_kind<1, ZT, SPR>(Z, R, rows, k, N, Gf, kp, scal, bound, flag, sms, sub, s);
-    else
-        launch_update_tc_kind<2, ZT, SPR>(Z, R, rows, k, N, Gf, kp, scal, bound, flag, sms, sub, s);
-}
-}  // namespace
-
-template <typename ZT>
-void launch_update_tc(ZT *Z, const float *R, int64_t rows, int k, const float *Gf, int kp, const double *scal,
-                      float bound, int *flag, cudaStream_t s) {
-    launch_update_tc_any<ZT, false>(Z, R, rows, k, Gf, kp, scal, bound, flag, UpdSub<ZT>{}, s);
-}
-template void launch_update_tc<float>(float *, const float *, int64_t, int, const float *, int, const double *, float,
-                                      int *, cudaStream_t);
-template void launch_update_tc<__nv_bfloat16>(__nv_bfloat16 *, const float *, int64_t, int, const float *, int,
-                                              const double *, float, int *, cudaStream_t);
-
-template <typename ZT>
-void launch_update_tc_subcsr(ZT *Z, const float *R, const SubCsr &sc, const ZT *Y, int64_t yrows, float alpha,
-                             int64_t rows, int k, const float *Gf, int kp, const double *scal, float bound, int *flag,
-                             cudaStream_t s) {
-    if (sc.rows != rows) throw ArgError{"launch_update_tc_subcsr: the sub-CSR has other rows"};
-    const UpdSub<ZT> sub{sc.ptr, sc.col[sc.cur], sc.val[sc.cur], Y, yrows, alpha};
-    launch_update_tc_any<ZT, true>(Z, R, rows, k, Gf, kp, scal, bound, flag, sub, s);
-}
-template void launch_update_tc_subcsr<float>(float *, const float *, const SubCsr &, const float *, int64_t, float,
-                                             int64_t, int, const float *, int, const double *, float, int *,
-                                             cudaStream_t);
-template void launch_update_tc_subcsr<__nv_bfloat16>(__nv_bfloat16 *, const float *, const SubCsr &,
-                                                     const __nv_bfloat16 *, int64_t, float, int64_t, int,
-                                                     const float *, int, const double *, float, int *, cudaStream_t);
-
-void bounds_report_tc(int reset, int64_t out[3]) {
-#ifdef DSANLS_BOUNDS
-    bounds_read_tu(reset, out);
-#else
-    (void)reset;
-    out[0] = out[1] = out[2] = 0;
-#endif
-}
-
 void set_tc_wait_debug(unsigned long long wait_ns, int starve) {
     DSANLS_CUDA(cudaMemcpyToSymbol(g_wait_ns, &wait_ns, sizeof(wait_ns)));
     DSANLS_CUDA(cudaMemcpyToSymbol(g_starve, &starve, sizeof(starve)));
 }
 
 void prime_tc_attributes(int max_smem) {
-    allow_max_dynamic_smem(k_update_tc<1, float, false>, max_smem);
-    allow_max_dynamic_smem(k_update_tc<2, float, false>, max_smem);
-    allow_max_dynamic_smem(k_update_tc<1, __nv_bfloat16, false>, max_smem);
-    allow_max_dynamic_smem(k_update_tc<2, __nv_bfloat16, false>, max_smem);
-    allow_max_dynamic_smem(k_update_tc<1, float, true>, max_smem);
-    allow_max_dynamic_smem(k_update_tc<2, float, true>, max_smem);
-    allow_max_dynamic_smem(k_update_tc<1, __nv_bfloat16, true>, max_smem);
-    allow_max_dynamic_smem(k_update_tc<2, __nv_bfloat16, true>, max_smem);
     allow_max_dynamic_smem(k_tc_gemm<4, true, false>, max_smem);
     allow_max_dynamic_smem(k_tc_gemm<3, true, false>, max_smem);
     allow_max_dynamic_smem(k_tc_gemm<4, false, false>, max_smem);

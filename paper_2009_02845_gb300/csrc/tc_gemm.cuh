@@ -95,6 +95,7 @@ void launch_transpose_bf16(const float *in, int64_t rows, int64_t cols, __nv_bfl
 // products, accurate to about binary32); entries clamped at `bound` when > 0;
 // NaN/Inf set bit 1 of *flag, a bounded wait that gives up bit 2.
 bool update_tc_supported(int k);
+void prime_update_attributes(int max_smem);
 // Z of type float, or bf16 for the bf16-factor form (z exact in bf16: three products;
 // the binary32 step rounded to bf16 when stored).
 template <typename ZT>
