@@ -710,8 +710,14 @@ __global__ void kb_sketch_t(const BatchInst *__restrict__ inst, int side, const 
     const uint32_t q4 = (uint32_t)(Kp >> 2), total = q4 * (uint32_t)dd;
     const float scale = b.scale[side];
     __nv_bfloat16 *St = St_all + st_off(b, side);
-    for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-        const uint32_t j = idx / q4, q = idx - j * q4;
+    // block idx is (column j, row block q) = idx divided by q4; the stride is divided once
+    const uint32_t stride = gridDim.x * blockDim.x, dj = stride / q4, dq = stride - dj * q4;
+    uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x, j = idx / q4, q = idx - j * q4;
+    for (; idx < total; idx += stride, j += dj, q += dq) {
+        if (q >= q4) {
+            q -= q4;
+            ++j;
+        }
         float z[4];
         gaussian4(b.seed, (uint32_t)side, t, q, j, z);
         __nv_bfloat16 o[4];

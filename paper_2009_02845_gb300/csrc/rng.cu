@@ -35,6 +35,15 @@ __global__ void k_field_words(uint64_t seed, uint32_t sid, uint64_t t, int64_t r
 }
 
 // t is read from device memory when t_dev != nullptr (graph replays).
+// A transposed block leaves in one store of 16 (8) bytes when the rows are a multiple of 4
+// (every column then starts on that many bytes), else element by element.
+DSANLS_DEV uint2 bf16x4(const float z[4]) {
+    return make_uint2((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(z[0])) |
+                          ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(z[1])) << 16),
+                      (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(z[2])) |
+                          ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(z[3])) << 16));
+}
+
 template <bool TRANSPOSED, typename OutT, int KIND>
 __global__ void k_gaussian_field(uint64_t seed, uint32_t sid, uint64_t t_host, const int64_t *t_dev,
                                  int64_t rows, int64_t cols, float scale, const int32_t *hcols, OutT *out) {
@@ -72,6 +81,8 @@ __global__ void k_gaussian_field(uint64_t seed, uint32_t sid, uint64_t t_host, c
         OutT *dst = out + j * rows + i0;
         if (sizeof(OutT) == 4 && i0 + 3 < rows && (rows & 3) == 0) {
             *reinterpret_cast<float4 *>(dst) = make_float4(z[0], z[1], z[2], z[3]);
+        } else if (sizeof(OutT) == 2 && (rows & 3) == 0) {
+            *reinterpret_cast<uint2 *>(dst) = bf16x4(z);
         } else {
 #pragma unroll
             for (int r = 0; r < 4; ++r)
@@ -104,6 +115,16 @@ __global__ void k_gaussian_dual(uint64_t seed, uint32_t sid, const int64_t *t_de
     float z[4];
     unit_draw4<KIND>(seed, sid, t, (uint32_t)q, (uint32_t)j, (uint32_t)cols, hcols, z);
     const int64_t i0 = 4 * q;
+    if ((rows & 3) == 0) {
+        const float zs[4] = {__fmul_rn(z[0], scale), __fmul_rn(z[1], scale), __fmul_rn(z[2], scale),
+                             __fmul_rn(z[3], scale)};
+        *reinterpret_cast<uint2 *>(out_b + j * rows + i0) = bf16x4(zs);
+        uint32_t w = 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) w |= (uint32_t)__nv_fp8_e4m3(z[r]).__x << (8 * r);
+        *reinterpret_cast<uint32_t *>(out_q + j * rows + i0) = w;
+        return;
+    }
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         if (i0 + r < rows) {
