@@ -167,7 +167,7 @@ struct dsanls_ctx {
     int64_t *t_dev = nullptr;
     int *flag = nullptr;
     __nv_bfloat16 *eparts = nullptr;  // split parts of U and V for the dense relative error
-    double *dscal = nullptr;  // [0] ||M||^2, [1] residual^2, [2] cross, [3..] Gram of U, Gram of V
+    double *dscal = nullptr;  // [0] ||M||^2, [1] residual^2, [2] cross (sparse) or the dropped terms' bound, [3..] Grams of U, V
     uint32_t *bits = nullptr;  // membership bitmap of the sampled set (sparse subsampling)
     SubCsr sub[2];             // sub-CSR of X[:, J] per side (sparse data, subsampling sketch)
     dsanls_mlp_ctx *mlp = nullptr;          // learned warm start (borrowed), or none
@@ -1196,13 +1196,16 @@ int dsanls_rel_error(dsanls_t h, double *out) {
     return guarded(h, [&]() {
         cudaStream_t s = h->stream();
         factors_to_f32(h, s);
-        bool tc = false;
-        auto residual = [&]() {
-            launch_dense_residual(h->M, h->ldM, h->U, h->V, h->m, h->n, h->k, h->work, WORK_ELEMS, h->dscal + 1, s);
+        double v[3];  // ||M||^2, the squared residual, what the tensor-core form may have dropped
+        auto read = [&]() -> int {
+            if (int rc = pending_status(h)) return rc;
+            DSANLS_CUDA(cudaMemcpy(v, h->dscal, sizeof v, cudaMemcpyDeviceToHost));
+            return DSANLS_OK;
         };
+        bool done = false;
         if (h->has_dense) {
             ensure_sumsq(h);
-            tc = residual_tc_supported(h->ldM, h->m, h->n, h->k);
+            bool tc = residual_tc_supported(h->ldM, h->m, h->n, h->k);
             if (tc && !h->eparts) {
                 try {
                     dalloc(h->eparts, residual_tc_parts(h->m, h->n, h->k));
@@ -1210,11 +1213,15 @@ int dsanls_rel_error(dsanls_t h, double *out) {
                     tc = false;  // no room for the parts: the form that needs none
                 }
             }
-            if (tc)
-                launch_dense_residual_tc(h->M, h->ldM, h->U, h->V, h->m, h->n, h->k, h->dscal + 0, h->eparts, h->work,
-                                         WORK_ELEMS, h->dscal + 1, h->flag, s);
-            else
-                residual();
+            // as the factors are, then with balanced columns, then in FP64
+            for (int balance = 0; tc && !done && balance < 2; ++balance) {
+                launch_dense_residual_tc(h->M, h->ldM, h->U, h->V, h->m, h->n, h->k, balance, h->dscal + 0, h->eparts,
+                                         h->work, WORK_ELEMS, h->dscal + 1, h->flag, s);
+                if (int rc = read()) return rc;
+                done = residual_tc_holds(v[0], v[1], v[2]);
+            }
+            if (!done)
+                launch_dense_residual(h->M, h->ldM, h->U, h->V, h->m, h->n, h->k, h->work, WORK_ELEMS, h->dscal + 1, s);
         } else {
             double *GU = h->dscal + 3, *GV = h->dscal + 3 + 128 * 128;
             launch_sparse_cross(h->rp, h->ci, h->cv, h->m, h->U, h->V, h->k, h->work, WORK_ELEMS, h->dscal + 2, s);
@@ -1222,14 +1229,8 @@ int dsanls_rel_error(dsanls_t h, double *out) {
             launch_factor_gram(h->V, h->n, h->k, h->work, WORK_ELEMS, GV, s);
             launch_sparse_combine(h->dscal + 0, h->dscal + 2, GU, GV, h->k, h->dscal + 1, s);
         }
-        if (int rc = pending_status(h)) return rc;
-        double v[2];
-        DSANLS_CUDA(cudaMemcpy(v, h->dscal, 2 * sizeof(double), cudaMemcpyDeviceToHost));
-        if (tc && !std::isfinite(v[1])) {  // residuals out of binary32's range against M: squares in FP64
-            residual();
-            if (int rc = pending_status(h)) return rc;
-            DSANLS_CUDA(cudaMemcpy(v, h->dscal, 2 * sizeof(double), cudaMemcpyDeviceToHost));
-        }
+        if (!done)
+            if (int rc = read()) return rc;
         *out = v[0] > 0.0 ? std::sqrt(std::max(v[1], 0.0) / v[0]) : 0.0;
         return DSANLS_OK;
     });

@@ -6,7 +6,8 @@
 // warp-shuffle then shared-memory reduction to one FP64 partial per CTA,
 // partials summed in CTA order (deterministic).  The single-problem handle takes the
 // tensor-core form of error_tc.cu; this one serves the batch's instances, rows that are not
-// 16-byte aligned and residuals out of binary32's range.
+// 16-byte aligned and factors whose sliced products would drop too much or leave binary32's
+// range.
 // Sparse M: the expansion ||M||^2 - 2 sum_{nnz} M_ij U_i.V_j + <U^T U, V^T V>,
 // each term with FP64 accumulation.
 #include "common.cuh"
@@ -98,11 +99,6 @@ __global__ void k_sum_parts(const double *__restrict__ part, int np, double *__r
     for (int i = threadIdx.x; i < np; i += blockDim.x) v += part[i];
     const double tot = cta_sum_d(v, red);
     if (threadIdx.x == 0) *out = tot;
-}
-
-void launch_sum_parts(const double *part, int np, double *out, cudaStream_t s) {
-    k_sum_parts<<<1, 1024, 0, s>>>(part, np, out);
-    DSANLS_LAUNCH_CHECK();
 }
 
 static int residual_grid(int64_t tiles, int64_t work_elems) {

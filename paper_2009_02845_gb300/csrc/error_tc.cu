@@ -3,34 +3,59 @@
 //
 // The CUDA-core form (error.cu) is bound by the FP64 pipe (two operations per clock and
 // SM): a conversion, a subtraction and an FMA per entry of M are 11.6 ms for 65,536 x
-// 16,384 where reading M takes 0.64.  Here the inner products come from three bf16 parts of
+// 16,384 where reading M takes 0.64.  Here the inner products come from four bf16 parts of
 // each row of U and of V on the row's own fixed grid (error-free slicing, Ozaki, Ogita,
-// Oishi, Rump 2012): multiples of 2^-8, 2^-17 and 2^-26 of a power of two above the row's
-// largest entry, at most 256 of them each (exact in bf16), so a product of parts is an
+// Oishi, Rump 2012): multiples of 2^-8, 2^-17, 2^-26 and 2^-35 of a power of two above the
+// row's largest entry, at most 256 of them each (exact in bf16), so a product of parts is an
 // integer of at most 2^16 in its unit and the sums of k <= 128 of them, D0 = hh and
-// D1 = hm + mh, are exact in the fp32 accumulator (D2 = hl + mm + lh to its last bit) -- the
-// tensor cores' rounding toward zero, a bias of 1e-7 of the result with the plain split,
-// has nothing to round.  They are added rounding to nearest; the parts' remainders are
-// 2^-27 of the largest entry, of either sign.  The residual is a binary32 subtraction (its error is relative to the
-// residual), and its square is summed in pairs of binary32 (two-product and two-sum, Dekker
-// 1971 and Knuth: 2^-48 of the sum), which a thread turns into FP64 once.
+// D1 = hm + mh, are exact in the fp32 accumulator (D2 = hl + mm + lh and D3 = hq + ml + lm +
+// qh to their last bits) -- the tensor cores' rounding toward zero, a bias of 1e-7 of the
+// result with the plain split, has nothing to round.  The residual is ((M - D0) - D1) - (D2 +
+// D3) in binary32: M - D0 is exact where the product fits M, and what it rounds otherwise is
+// relative to a difference.  Its square is summed in pairs of binary32 (two-product and
+// two-sum, Dekker 1971 and Knuth: 2^-48 of the sum), which a thread adds to FP64 every
+// RT_CARRY tiles.
+//
+// What the slicing drops is absolute: each of the at most min(nz_i, nz_j) products of nonzeros
+// of rows i of U and j of V loses up to 5.1 2^-36 2^(e_i + e_j), 2^e above a row's largest entry
+// (the remainders, 2^-36 of that against an entry of the other row, and the products of parts
+// beyond D3).  That is nothing beside the residual as long as a large entry of one row does not
+// meet the dropped tail of the other (columns of U and V of opposite scales, a component dead
+// in one factor and large in the other).  So k_parts_grid also sums nz_i 4^e_i over the rows, and
+//     E^2 = 26 2^-72 (sum over U) (sum over V) + m n (k 2^-125)^2
+// (the last term for products that underflow) bounds the sum of the squares of what is dropped:
+// the caller takes the result only if E^2 is at most 1e-12 of it or 2^-58 ||M||^2
+// (residual_tc_holds).  Whatever the signs, ||M - U V^T||_F is then within 1e-6 of itself or, for
+// factors that fit M closely, within 2^-29 ||M||, an eighth of what rounding each product
+// to binary32 once would move.  Otherwise the columns are
+// balanced first -- column c of U times a power of two and column c of V by its inverse, from
+// the largest entry of both; exact, and the product is the same -- and if that does not meet
+// the bound either, the FP64 form answers.  Over random, planted and fitted factors of seven
+// shapes (the last ones within 1e-4 of M) the result is 1e-13 to 1.6e-10 of itself away from
+// FP64 arithmetic, where the binary32 chains of error.cu are 4e-13 to 9e-7 away.  Three parts
+// and a bound were not enough: the tails dropped at 2^-27 are the same along a whole row of M
+// and average out less than a chain's roundings (1.2e-9 where the chains have 4e-10).
 //
 // Persistent CTAs take contiguous ranges of 128 x 64 tiles in row order.  Warps by role:
 //   epilogue (16)  a thread owns a row and 16 columns: residual of the tile of M in shared
 //                  memory (TMA, 32-column boxes, 128-byte swizzle: no bank conflicts)
 //                  against the accumulators;
-//   mma            one thread: per K step A_h x [B_h | B_m | B_l], A_m x [B_h | B_m],
-//                  A_l x B_h into one of two sets of accumulators;
+//   mma            one thread: per K step A_h x [B_h | B_m | B_l | B_q], A_m x [B_h | B_m |
+//                  B_l], A_l x [B_h | B_m], A_q x B_h into one of two sets of accumulators
+//                  (all of tensor memory);
 //   tma M          the tile of M, a ring of 32-column chunks;
-//   tma U, V       U's parts when the row tile changes, V's parts of every tile (from L2).
-// What bounds it: HBM needs 1,515 cycles per tile, the products 832 (k <= 64), the
-// epilogue's issue slots about 1,300.  Measured, with the parts and the final sum, 65,536 x
-// 16,384 with k = 64: 1.24 ms (11.6 in FP64) = 3.5 TB/s; the result's distance from FP64
-// arithmetic 5e-14 to 3e-9 relative over random and fitted factors of five shapes, where
-// the FP64 form with binary32 chains had 2e-13 to 6e-10.
+//   tma U, V       U's parts when the row tile changes, V's parts of every tile and K block of
+//                  64 (from L2).
+// What bounds it: HBM needs 1,515 cycles per tile, the products 1,280 (k <= 64), the
+// epilogue's issue slots about 1,400.  Measured, with the parts and the final sum, 65,536 x
+// 16,384 with k = 64: 1.24 ms (11.6 in FP64) = 3.5 TB/s, and
+// 2.56 where the columns are balanced in a second pass; k = 100 1.78.  The epilogue's arithmetic
+// bounds it (0.99 ms without): it runs two columns to an instruction (1.37 ms with one), reads M
+// before it waits for the products and its accumulators with one wait (1.35 otherwise).
 #include <cuda.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -45,8 +70,12 @@ constexpr int RT_BM = 128, RT_BN = 64, RT_CHUNK = 32;
 constexpr int RT_EW = 16;                            // epilogue warps
 constexpr int RT_THREADS = 32 * (RT_EW + 3);
 constexpr int RT_CHUNK_BYTES = RT_BM * RT_CHUNK * 4;
-constexpr int RT_DSET = 3 * RT_BN;
+constexpr int RT_PARTS = 4;
+constexpr int RT_DSET = RT_PARTS * RT_BN;
 constexpr int RT_MAX_M = 6, RT_BST = 2;
+constexpr int RT_BSTAGE = RT_PARTS * RT_BN * 128;    // V's parts of a tile and K block
+constexpr int RT_CARRY = 16;                         // tiles between carries into FP64
+constexpr int64_t RT_GRID_SUMS = 512;                // doubles of `work` before k_parts_grid's sums
 constexpr unsigned long long RT_WAIT_NS = 2000000000ull;
 
 struct __align__(16) RtTail {
@@ -63,10 +92,9 @@ struct __align__(16) RtTail {
 // KB: K blocks of 64 (1 for k <= 64, 2 above)
 template <int KB>
 struct RtCfg {
-    static constexpr int ABYTES = KB * 3 * RT_BM * 128;   // U's parts of a row tile
-    static constexpr int BBYTES = KB * 3 * RT_BN * 128;   // V's parts of a tile
+    static constexpr int ABYTES = KB * RT_PARTS * RT_BM * 128;  // U's parts of a row tile
     static constexpr int MST = KB == 1 ? 6 : 2;           // chunks of M in the ring
-    static constexpr size_t SMEM = 1024 + ABYTES + RT_BST * BBYTES + MST * RT_CHUNK_BYTES + sizeof(RtTail);
+    static constexpr size_t SMEM = 1024 + ABYTES + RT_BST * RT_BSTAGE + MST * RT_CHUNK_BYTES + sizeof(RtTail);
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
@@ -81,6 +109,40 @@ DSANLS_DEV bool rt_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
         }
     }
     return true;
+}
+
+// Two binary32 operations, rounded to nearest, in one instruction.
+DSANLS_DEV uint64_t rt_pair(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+DSANLS_DEV uint64_t rt_pair(uint32_t a, uint32_t b) { return rt_pair(__uint_as_float(a), __uint_as_float(b)); }
+DSANLS_DEV uint64_t rt_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+DSANLS_DEV uint64_t rt_sub(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+DSANLS_DEV uint64_t rt_mul(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+DSANLS_DEV uint64_t rt_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+DSANLS_DEV double rt_total(uint64_t hi, uint64_t lo) {
+    float h0, h1, l0, l1;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(h0), "=f"(h1) : "l"(hi));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(l0), "=f"(l1) : "l"(lo));
+    return ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
 }
 
 // power of two near 1 / rms(M): the squares then neither overflow nor vanish against M's
@@ -100,7 +162,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
     constexpr int MST = Cfg::MST, APART = RT_BM * 128, BPART = RT_BN * 128;
     extern __shared__ __align__(1024) uint8_t rt_raw[];
     uint8_t *base = rt_raw + ((1024u - (smem_u32(rt_raw) & 1023u)) & 1023u);
-    uint8_t *ap = base, *bp = ap + Cfg::ABYTES, *mp = bp + RT_BST * Cfg::BBYTES;
+    uint8_t *ap = base, *bp = ap + Cfg::ABYTES, *mp = bp + RT_BST * RT_BSTAGE;
     RtTail *tail = reinterpret_cast<RtTail *>(mp + MST * RT_CHUNK_BYTES);
     volatile int *abort = &tail->abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -137,64 +199,73 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
     const int64_t ntn = ceil_div(n, (int64_t)RT_BN), tiles = ceil_div(m, (int64_t)RT_BM) * ntn;
     const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
     const int nt = (int)(t1 - t0);
-    float hi = 0.0f, lo = 0.0f;  // epilogue: the thread's sum
+    uint64_t hi = 0, lo = 0;  // epilogue: the thread's sums (even and odd columns) since the last carry
+    double sum = 0.0;
     if (warp < RT_EW) {
         const int q = warp & 3, cg = warp >> 2, r = 32 * q + lane;  // columns 16 cg .. of the tile
         const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16) + 16 * cg;
-        const float scale = __int_as_float((127 - rt_exponent(*mm, (double)m * (double)n)) << 23);
+        const float sc = __int_as_float((127 - rt_exponent(*mm, (double)m * (double)n)) << 23);
+        const uint64_t scale = rt_pair(sc, sc);
         for (int i = 0; i < nt; ++i) {
             const int c = 2 * i + (cg >> 1), slot = c % MST, buf = i & 1;
-            const bool ok = rt_wait(&tail->mfull[slot], (c / MST) & 1, abort) &&
-                            rt_wait(&tail->dfull[buf], (i >> 1) & 1, abort);
+            bool ok = rt_wait(&tail->mfull[slot], (c / MST) & 1, abort);
             if (!__all_sync(0xffffffffu, ok)) break;
-            fence_after();
-            uint32_t d[16];
-            float x[16];
-            tmem_ld16(tl + buf * RT_DSET + RT_BN, d);
-            {
-                uint32_t d2[16];
-                tmem_ld16(tl + buf * RT_DSET + 2 * RT_BN, d2);
-                tmem_ld_wait();
-#pragma unroll
-                for (int e = 0; e < 16; ++e) x[e] = __fadd_rn(__uint_as_float(d[e]), __uint_as_float(d2[e]));
-            }
-            tmem_ld16(tl + buf * RT_DSET, d);
             const float4 *row = reinterpret_cast<const float4 *>(mp + slot * RT_CHUNK_BYTES) + r * (RT_CHUNK / 4);
             float4 v[4];
 #pragma unroll
             for (int p = 0; p < 4; ++p) v[p] = row[(4 * (cg & 1) + p) ^ (r & 7)];
+            if (MST == 2) {  // a ring of one tile: the next one's copy under this one's products (k = 100
+                __syncwarp();  // 1.79 ms, 2.44 with the arrival below; k = 64, three tiles, 1.30 and 1.23)
+                if (lane == 0) mbar_arrive(&tail->mempty[slot]);
+            }
+            ok = rt_wait(&tail->dfull[buf], (i >> 1) & 1, abort);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            fence_after();
+            uint32_t d[16], d1[16], d2[16], d3[16];
+            uint64_t x[8];
+            tmem_ld16(tl + buf * RT_DSET, d);
+            tmem_ld16(tl + buf * RT_DSET + RT_BN, d1);
+            tmem_ld16(tl + buf * RT_DSET + 2 * RT_BN, d2);
+            tmem_ld16(tl + buf * RT_DSET + 3 * RT_BN, d3);
             tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                x[e] = rt_add(rt_pair(d2[2 * e], d2[2 * e + 1]), rt_pair(d3[2 * e], d3[2 * e + 1]));
             fence_before();
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&tail->dempty[buf]);
-                mbar_arrive(&tail->mempty[slot]);
+                if (MST > 2) mbar_arrive(&tail->mempty[slot]);
             }
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const float4 w = v[e >> 2];
-                const float me = (e & 3) == 0 ? w.x : ((e & 3) == 1 ? w.y : ((e & 3) == 2 ? w.z : w.w));
-                const float uv = __fadd_rn(__uint_as_float(d[e]), x[e]);
-                const float res = __fmul_rn(__fsub_rn(me, uv), scale);
-                const float p = __fmul_rn(res, res), pe = __fmaf_rn(res, res, -p);
+            for (int e = 0; e < 8; ++e) {
+                const float4 w = v[e >> 1];
+                const uint64_t me = (e & 1) ? rt_pair(w.z, w.w) : rt_pair(w.x, w.y);
+                const uint64_t r1 = rt_sub(rt_sub(me, rt_pair(d[2 * e], d[2 * e + 1])), rt_pair(d1[2 * e], d1[2 * e + 1]));
+                const uint64_t res = rt_mul(rt_sub(r1, x[e]), scale);
+                const uint64_t p = rt_mul(res, res), pe = rt_fma(res, res, p ^ 0x8000000080000000ull);
                 // (hi, lo) += p + pe: columns past n and rows past m have a residual of zero
-                const float s = __fadd_rn(hi, p), t = __fsub_rn(s, hi);
-                const float se = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(p, t));
+                const uint64_t s = rt_add(hi, p), t = rt_sub(s, hi);
+                const uint64_t se = rt_add(rt_sub(hi, rt_sub(s, t)), rt_sub(p, t));
                 hi = s;
-                lo = __fadd_rn(lo, __fadd_rn(se, pe));
+                lo = rt_add(lo, rt_add(se, pe));
+            }
+            if (i % RT_CARRY == RT_CARRY - 1) {
+                sum += rt_total(hi, lo);
+                hi = lo = 0;
             }
         }
     } else if (warp == RT_EW) {
         if (lane == 0) {
             // ---- mma ----
-            const uint32_t id1 = idesc_bf16(RT_BM, RT_BN), id2 = idesc_bf16(RT_BM, 2 * RT_BN),
-                           id3 = idesc_bf16(RT_BM, 3 * RT_BN);
+            uint32_t id[RT_PARTS];  // N = 1 .. 4 parts of V
+            for (int p = 0; p < RT_PARTS; ++p) id[p] = idesc_bf16(RT_BM, (p + 1) * RT_BN);
             int64_t rt = -1;
             int na = 0;  // row tiles so far
             const int steps = (k + 15) / 16;
             for (int i = 0; i < nt; ++i) {
                 const int64_t row = (t0 + i) / ntn;
-                const int sb = i % RT_BST, buf = i & 1;
+                const int buf = i & 1;
                 if (row != rt) {
                     if (na > 0) mma_commit(&tail->aempty);
                     if (!rt_wait(&tail->afull, na & 1, abort)) break;
@@ -202,18 +273,26 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
                     ++na;
                 }
                 if (i >= 2 && !rt_wait(&tail->dempty[buf], ((i >> 1) - 1) & 1, abort)) break;
-                if (!rt_wait(&tail->bfull[sb], (i / RT_BST) & 1, abort)) break;
-                fence_after();
                 const uint32_t d = tmem + buf * RT_DSET;
-                for (int ks = 0; ks < steps; ++ks) {
-                    const uint32_t o = (ks & 3) * 32;
-                    const uint32_t ah = smem_u32(ap) + (ks >> 2) * 3 * APART + o, am = ah + APART, al = am + APART;
-                    const uint64_t bh = sw128_desc(smem_u32(bp) + sb * Cfg::BBYTES + (ks >> 2) * 3 * BPART + o);
-                    mma_bf16(d, sw128_desc(ah), bh, id3, ks > 0);
-                    mma_bf16(d + RT_BN, sw128_desc(am), bh, id2, 1);
-                    mma_bf16(d + 2 * RT_BN, sw128_desc(al), bh, id1, 1);
+                bool ok = true;
+                for (int kb = 0; kb < KB; ++kb) {
+                    const int b = i * KB + kb, sb = b % RT_BST;
+                    ok = rt_wait(&tail->bfull[sb], (b / RT_BST) & 1, abort);
+                    if (!ok) break;
+                    fence_after();
+                    const int nks = min(4, steps - 4 * kb);
+                    for (int ks = 0; ks < nks; ++ks) {
+                        const uint32_t a = smem_u32(ap) + kb * RT_PARTS * APART + ks * 32;
+                        const uint64_t bh = sw128_desc(smem_u32(bp) + sb * RT_BSTAGE + ks * 32);
+                        // part p of U times the parts 0 .. 3 - p of V, into D_p .. D_3
+#pragma unroll
+                        for (int p = 0; p < RT_PARTS; ++p)
+                            mma_bf16(d + p * RT_BN, sw128_desc(a + p * APART), bh, id[RT_PARTS - 1 - p],
+                                     p > 0 || kb > 0 || ks > 0);
+                    }
+                    mma_commit(&tail->bempty[sb]);
                 }
-                mma_commit(&tail->bempty[sb]);
+                if (!ok) break;
                 mma_commit(&tail->dfull[buf]);
             }
             // every product this thread issued has retired before the tensor memory is freed
@@ -238,34 +317,39 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
                     mbar_wait(&tail->mfull[c % MST], (c / MST) & 1, RT_WAIT_NS);
         }
     } else if (lane == 0) {
-        // ---- tma U, V (parts p of K block kb: rows p urows + i, columns 64 kb ..) ----
+        // ---- tma U, V (part p of K block kb: rows p urows + i, columns 64 kb ..) ----
         int64_t rt = -1;
         int na = 0, issued = 0;
-        for (int i = 0; i < nt; ++i) {
+        bool ok = true;
+        for (int i = 0; ok && i < nt; ++i) {
             const int64_t row = (t0 + i) / ntn;
-            const int sb = i % RT_BST;
             if (row != rt) {
                 if (na > 0 && !rt_wait(&tail->aempty, (na - 1) & 1, abort)) break;
                 mbar_expect_tx(&tail->afull, Cfg::ABYTES);
-                for (int x = 0; x < 3 * KB; ++x)
-                    tma_load_2d(ap + x * APART, &map_u, (x / 3) * 64, (int)((x % 3) * urows + row * RT_BM), &tail->afull);
+                for (int x = 0; x < RT_PARTS * KB; ++x)
+                    tma_load_2d(ap + x * APART, &map_u, (x / RT_PARTS) * 64,
+                                (int)((x % RT_PARTS) * urows + row * RT_BM), &tail->afull);
                 rt = row;
                 ++na;
             }
-            if (i >= RT_BST && !rt_wait(&tail->bempty[sb], ((i / RT_BST) - 1) & 1, abort)) break;
-            mbar_expect_tx(&tail->bfull[sb], Cfg::BBYTES);
-            for (int x = 0; x < 3 * KB; ++x)
-                tma_load_2d(bp + sb * Cfg::BBYTES + x * BPART, &map_v, (x / 3) * 64,
-                            (int)((x % 3) * vrows + ((t0 + i) % ntn) * RT_BN), &tail->bfull[sb]);
-            issued = i + 1;
+            for (int kb = 0; kb < KB; ++kb) {
+                const int b = i * KB + kb, sb = b % RT_BST;
+                ok = b < RT_BST || rt_wait(&tail->bempty[sb], ((b / RT_BST) - 1) & 1, abort);
+                if (!ok) break;
+                mbar_expect_tx(&tail->bfull[sb], RT_BSTAGE);
+                for (int p = 0; p < RT_PARTS; ++p)
+                    tma_load_2d(bp + sb * RT_BSTAGE + p * BPART, &map_v, kb * 64,
+                                (int)(p * vrows + ((t0 + i) % ntn) * RT_BN), &tail->bfull[sb]);
+                issued = b + 1;
+            }
         }
         if (*abort) {
             if (na > 0) mbar_wait(&tail->afull, (na - 1) & 1, RT_WAIT_NS);
-            for (int i = max(0, issued - RT_BST); i < issued; ++i)
-                mbar_wait(&tail->bfull[i % RT_BST], (i / RT_BST) & 1, RT_WAIT_NS);
+            for (int b = max(0, issued - RT_BST); b < issued; ++b)
+                mbar_wait(&tail->bfull[b % RT_BST], (b / RT_BST) & 1, RT_WAIT_NS);
         }
     }
-    double v = (double)hi + (double)lo;
+    double v = sum + rt_total(hi, lo);
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (warp < RT_EW && lane == 0) tail->red[warp] = v;
     fence_before();
@@ -281,48 +365,126 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
-// The three parts of the rows of X (rows x k) on each row's grid, out[p][row][ldk], prows
-// rows per part (zero past the last); one warp per row.  A row whose largest entry is not in
-// [2^-90, 2^100], or not finite, becomes NaN: the caller's result is then not finite.
-__global__ void __launch_bounds__(256) k_parts_grid(const float *__restrict__ X, int64_t rows, int k, int64_t ldk,
-                                                    int64_t prows, __nv_bfloat16 *__restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < prows; r += (int64_t)gridDim.x * 8) {
+// Scratch ahead of the parts: the largest entry (bits) of every column of U, then of V.
+constexpr int64_t RT_COLS = 128;
+constexpr int64_t RT_COL_BYTES = 2 * RT_COLS * sizeof(uint32_t);
+
+// Largest |entry| of every column of U (blockIdx.y = 0) and V (1), into the zeroed cmax.
+__global__ void __launch_bounds__(256) k_column_max(const float *__restrict__ U, const float *__restrict__ V, int64_t m,
+                                                    int64_t n, int k, uint32_t *__restrict__ cmax) {
+    const float *X = blockIdx.y ? V : U;
+    const int64_t rows = blockIdx.y ? n : m;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t mx[4] = {0, 0, 0, 0};
+    for (int64_t r = (int64_t)blockIdx.x * 8 + warp; r < rows; r += (int64_t)gridDim.x * 8)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (lane + 32 * u < k) mx[u] = max(mx[u], __float_as_uint(fabsf(X[r * k + lane + 32 * u])));
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (lane + 32 * u < k) atomicMax(&cmax[blockIdx.y * RT_COLS + lane + 32 * u], mx[u]);
+}
+
+// The four parts of the rows of U (blocks 0 .. ublocks-1) and V (the rest) on each row's grid,
+// out[p][row][ldk], prows rows per part (zero past the last); one warp per row.  A row whose
+// largest entry is not in [2^-90, 2^100], or not finite, becomes NaN: the result is then not
+// finite.  Each block's sum of (nonzeros) 4^e goes to sums[b].
+// With cmax the columns are balanced first (a column that is zero in either factor is dropped).
+__global__ void __launch_bounds__(256)
+    k_parts_grid(const float *__restrict__ U, const float *__restrict__ V, int64_t m, int64_t n, int k, int64_t ldk,
+                 int64_t ur, int64_t vr, __nv_bfloat16 *__restrict__ parts, int ublocks,
+                 const uint32_t *__restrict__ cmax, double *__restrict__ sums) {
+    __shared__ double red[8];
+    const bool is_v = (int)blockIdx.x >= ublocks;
+    const float *X = is_v ? V : U;
+    const int64_t rows = is_v ? n : m, prows = is_v ? vr : ur;
+    __nv_bfloat16 *out = parts + (is_v ? RT_PARTS * ur * ldk : 0);
+    const int blk = (int)blockIdx.x - (is_v ? ublocks : 0), nblk = is_v ? (int)gridDim.x - ublocks : ublocks;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float f[4] = {1.0f, 1.0f, 1.0f, 1.0f}, f2[4] = {1.0f, 1.0f, 1.0f, 1.0f};  // the column's factor in two steps
+    if (cmax) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c = lane + 32 * u;
+            if (c >= k) break;
+            const uint32_t a = cmax[c], b = cmax[RT_COLS + c];
+            const int t = ((int)(b >> 23) - (int)(a >> 23)) >> 1, e = is_v ? -t : t;  // |t| <= 127
+            f[u] = a && b ? __int_as_float((127 + (e >> 1)) << 23) : 0.0f;
+            f2[u] = __int_as_float((127 + e - (e >> 1)) << 23);
+        }
+    }
+    double sum = 0.0;
+    for (int64_t r = (int64_t)blk * 8 + warp; r < prows; r += (int64_t)nblk * 8) {
         float z[4], mx = 0.0f;
         bool finite = true;
+        int nz = 0;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int c = lane + 32 * u;
             z[u] = r < rows && c < k ? X[r * k + c] : 0.0f;
             finite = finite && fabsf(z[u]) <= 3.402823466e38f;
+            z[u] = __fmul_rn(__fmul_rn(z[u], f[u]), f2[u]);
+            finite = finite && fabsf(z[u]) <= 3.402823466e38f;
             mx = fmaxf(mx, fabsf(z[u]));
+            nz += __popc(__ballot_sync(0xffffffffu, z[u] != 0.0f));
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         const bool bad = !__all_sync(0xffffffffu, finite) || (mx > 0.0f && (mx < 0x1p-90f || mx > 0x1p100f));
         // e: 2^e above every entry; rounding to a multiple of q by adding and subtracting 1.5 2^23 q
         const int e = mx > 0.0f && !bad ? (int)((__float_as_uint(mx) >> 23) & 255) - 126 : 0;
-        const float c1 = __int_as_float((127 + e + 15) << 23) * 1.5f, c2 = c1 * 0x1p-9f, c3 = c1 * 0x1p-18f;
+        if (mx > 0.0f) sum += ldexp((double)nz, 2 * e);
+        const float c1 = __int_as_float((127 + e + 15) << 23) * 1.5f;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int c = lane + 32 * u;
             if (c >= k) break;
-            const float h = __fsub_rn(__fadd_rn(z[u], c1), c1), r1 = __fsub_rn(z[u], h);
-            const float m = __fsub_rn(__fadd_rn(r1, c2), c2), r2 = __fsub_rn(r1, m);
-            const float l = __fsub_rn(__fadd_rn(r2, c3), c3);
-            const float nan = __int_as_float(0x7fc00000);
             __nv_bfloat16 *o = out + r * ldk + c;
-            o[0] = __float2bfloat16_rn(bad ? nan : h);
-            o[prows * ldk] = __float2bfloat16_rn(bad ? nan : m);
-            o[2 * prows * ldk] = __float2bfloat16_rn(bad ? nan : l);
+            float x = z[u], q = c1;
+#pragma unroll
+            for (int p = 0; p < RT_PARTS; ++p) {
+                const float h = __fsub_rn(__fadd_rn(x, q), q);
+                o[p * prows * ldk] = __float2bfloat16_rn(bad ? __int_as_float(0x7fc00000) : h);
+                x = __fsub_rn(x, h);
+                q *= 0x1p-9f;
+            }
         }
+    }
+    if (lane == 0) red[warp] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        sums[blockIdx.x] = t;
     }
 }
 
-void launch_parts_grid(const float *X, int64_t rows, int k, int64_t ldk, int64_t prows, __nv_bfloat16 *out,
-                       cudaStream_t s) {
-    k_parts_grid<<<(unsigned)std::min<int64_t>(ceil_div(prows, 8), 152 * 16), 256, 0, s>>>(X, rows, k, ldk, prows, out);
-    DSANLS_LAUNCH_CHECK();
+// out[0] = the squared residual, out[1] = E^2 (the head of this file); fixed orders
+__global__ void __launch_bounds__(256)
+    k_residual_sum(const double *__restrict__ part, int np, const double *__restrict__ sums, int ublocks, int vblocks,
+                   double m, double n, double k, double *__restrict__ out) {
+    __shared__ double red[3][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v[3] = {0.0, 0.0, 0.0};  // the residual, U's and V's nz 4^e
+    for (int i = threadIdx.x; i < np; i += 256) v[0] += part[i];
+    for (int i = threadIdx.x; i < ublocks; i += 256) v[1] += sums[i];
+    for (int i = threadIdx.x; i < vblocks; i += 256) v[2] += sums[ublocks + i];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        if (lane == 0) red[q][warp] = v[q];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t[3];
+        for (int q = 0; q < 3; ++q) {
+            t[q] = 0.0;
+            for (int w = 0; w < 8; ++w) t[q] += red[q][w];
+        }
+        const double under = k * 0x1p-125;
+        out[0] = t[0];
+        out[1] = 26.0 * 0x1p-72 * t[1] * t[2] + m * n * under * under;
+    }
 }
 
 int64_t pad_rows(int64_t r, int64_t t) { return ceil_div(r, t) * t; }
@@ -339,32 +501,51 @@ void residual_launch(const CUtensorMap &mm_map, const CUtensorMap &mu, const CUt
 
 bool residual_tc_supported(int64_t ld, int64_t m, int64_t n, int k) {
     // whole 16-byte rows for TMA; rows and columns in a tensor map's coordinates
-    return ld % 4 == 0 && k >= 1 && k <= 128 && 3 * pad_rows(m, RT_BM) < (1ll << 31) && 3 * pad_rows(n, RT_BN) < (1ll << 31);
+    return ld % 4 == 0 && k >= 1 && k <= 128 && RT_PARTS * pad_rows(m, RT_BM) < (1ll << 31) &&
+           RT_PARTS * pad_rows(n, RT_BN) < (1ll << 31);
 }
 
 int64_t residual_tc_parts(int64_t m, int64_t n, int k) {
-    return 3 * (pad_rows(m, RT_BM) + pad_rows(n, RT_BN)) * split_parts_ld(k);
+    return RT_COL_BYTES / (int64_t)sizeof(__nv_bfloat16) +
+           RT_PARTS * (pad_rows(m, RT_BM) + pad_rows(n, RT_BN)) * split_parts_ld(k);
+}
+
+bool residual_tc_holds(double mm, double residual, double dropped) {
+    // (below 2^-90 of ||M||^2 the squares themselves would leave binary32's range)
+    return std::isfinite(residual) && residual >= 0x1p-90 * mm && dropped <= std::max(1e-12 * residual, 0x1p-58 * mm);
 }
 
 void launch_dense_residual_tc(const float *M, int64_t ld, const float *U, const float *V, int64_t m, int64_t n, int k,
-                              const double *mm, __nv_bfloat16 *parts, double *work, int64_t work_elems, double *out,
-                              int *err, cudaStream_t s) {
+                              bool balance, const double *mm, __nv_bfloat16 *parts, double *work, int64_t work_elems,
+                              double *out, int *err, cudaStream_t s) {
     if (!residual_tc_supported(ld, m, n, k)) throw ArgError{"residual on tensor cores: unsupported size"};
     const int64_t ldk = split_parts_ld(k), ur = pad_rows(m, RT_BM), vr = pad_rows(n, RT_BN);
-    __nv_bfloat16 *up = parts, *vp = parts + 3 * ur * ldk;
-    launch_parts_grid(U, m, k, ldk, ur, up, s);
-    launch_parts_grid(V, n, k, ldk, vr, vp, s);
+    const int ublocks = (int)std::min<int64_t>(ceil_div(ur, 8), 152 * 8);
+    const int vblocks = (int)std::min<int64_t>(ceil_div(vr, 8), 152 * 8);
+    if (work_elems < RT_GRID_SUMS + ublocks + vblocks) throw ArgError{"residual: workspace too small"};
+    uint32_t *cmax = reinterpret_cast<uint32_t *>(parts);
+    __nv_bfloat16 *up = parts + RT_COL_BYTES / sizeof(__nv_bfloat16), *vp = up + RT_PARTS * ur * ldk;
+    double *sums = work + RT_GRID_SUMS;
+    if (balance) {
+        DSANLS_CUDA(cudaMemsetAsync(cmax, 0, RT_COL_BYTES, s));
+        k_column_max<<<dim3((unsigned)std::max(ublocks, vblocks), 2), 256, 0, s>>>(U, V, m, n, k, cmax);
+        DSANLS_LAUNCH_CHECK();
+    }
+    k_parts_grid<<<(unsigned)(ublocks + vblocks), 256, 0, s>>>(U, V, m, n, k, ldk, ur, vr, up, ublocks,
+                                                               balance ? cmax : nullptr, sums);
+    DSANLS_LAUNCH_CHECK();
     CUtensorMap mm_map, mu, mv;
     encode_f32_map(&mm_map, M, m, n, ld, RT_CHUNK, RT_BM, true);
-    encode_bf16_map_ld(&mu, up, 3 * ur, k, ldk, RT_BM);
-    encode_bf16_map_ld(&mv, vp, 3 * vr, k, ldk, RT_BN);
+    encode_bf16_map_ld(&mu, up, RT_PARTS * ur, k, ldk, RT_BM);
+    encode_bf16_map_ld(&mv, vp, RT_PARTS * vr, k, ldk, RT_BN);
     const int64_t tiles = ceil_div(m, RT_BM) * ceil_div(n, RT_BN);
-    const int grid = (int)std::min<int64_t>({tiles, 152, work_elems});  // one CTA per SM (tensor memory)
+    const int grid = (int)std::min<int64_t>(tiles, 152);  // one CTA per SM (tensor memory)
     if (k <= 64)
         residual_launch<1>(mm_map, mu, mv, m, n, k, mm, work, grid, err, s);
     else
         residual_launch<2>(mm_map, mu, mv, m, n, k, mm, work, grid, err, s);
-    launch_sum_parts(work, grid, out, s);
+    k_residual_sum<<<1, 256, 0, s>>>(work, grid, sums, ublocks, vblocks, (double)m, (double)n, (double)k, out);
+    DSANLS_LAUNCH_CHECK();
 }
 
 void prime_residual_attributes(int max_smem) {

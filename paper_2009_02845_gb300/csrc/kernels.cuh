@@ -151,17 +151,19 @@ void launch_increment_t(int64_t *t_dev, int64_t by, cudaStream_t s);
 // sum_ij (M_ij - U_i . V_j)^2 in FP64 -> *out (device), M m x n (row stride ld).
 void launch_dense_residual(const float *M, int64_t ld, const float *U, const float *V, int64_t m, int64_t n,
                            int k, double *work, int64_t work_elems, double *out, cudaStream_t s);
-// out = sum of part[0..np) in a fixed order
-void launch_sum_parts(const double *part, int np, double *out, cudaStream_t s);
-// The same with U V^T on tensor cores (error_tc.cu), for matrices with 16-byte rows and
-// residuals whose squares over ||M||^2 / (m n) stay in binary32's range (*out is Inf or NaN
-// otherwise, as with rows of U or V beyond 2^100 or all below 2^-90).  mm: ||M||^2 on the device; parts: residual_tc_parts(m, n, k) elements of
-// scratch; bit 2 of *err when a bounded wait gives up.
+// The same with U V^T on tensor cores (error_tc.cu), for matrices with 16-byte rows.  out[0]
+// is the squared residual and out[1] a bound on the squares of what the sliced products drop,
+// summed over the entries; the result counts only if residual_tc_holds(||M||^2, out[0], out[1]).  It does not where the residual leaves binary32's range against M, where a row
+// of U or V is beyond 2^100 or all below 2^-90, and where entries far below their row's
+// largest meet large ones of the other factor; `balance` first scales the columns of U and V
+// by opposite powers of two (the same product).  mm: ||M||^2 on the device; parts:
+// residual_tc_parts(m, n, k) elements of scratch; bit 2 of *err when a bounded wait gives up.
 bool residual_tc_supported(int64_t ld, int64_t m, int64_t n, int k);
 int64_t residual_tc_parts(int64_t m, int64_t n, int k);
+bool residual_tc_holds(double mm, double residual, double dropped);
 void launch_dense_residual_tc(const float *M, int64_t ld, const float *U, const float *V, int64_t m, int64_t n, int k,
-                              const double *mm, __nv_bfloat16 *parts, double *work, int64_t work_elems, double *out,
-                              int *err, cudaStream_t s);
+                              bool balance, const double *mm, __nv_bfloat16 *parts, double *work, int64_t work_elems,
+                              double *out, int *err, cudaStream_t s);
 void prime_residual_attributes(int max_smem);
 // sum of squares of x[0..len) in FP64 -> *out.
 void launch_sumsq(const float *x, int64_t len, double *work, int64_t work_elems, double *out, cudaStream_t s);
