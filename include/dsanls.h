@@ -233,13 +233,15 @@ int dsanls_kernel_launches(uint64_t *out);
  * switch off.  Never fails itself.
  *
  * dsanls_debug_tc_wait(wait_ns, starve), on the current device: wait_ns > 0
- * replaces the 2 s limit of the bounded waits of the tensor-core kernels
- * (0 restores it); starve = 1 (needs wait_ns > 0) makes the TMA producer of
- * the tensor-core GEMM issue no copy, so its consumers' waits run out with
- * nothing in flight: the kernel frees its tensor memory, returns, and the
- * next synchronising call of the handle reports DSANLS_ETIMEOUT.  EINVAL for
- * starve outside {0, 1} or starve without a limit; ECUDA if the device
- * symbols cannot be written.  Synchronous. */
+ * replaces the 2 s limit of the bounded waits of the handles' tensor-core
+ * kernels -- the products of every precision, the row update and the dense
+ * relative error (0 restores it; the batched form's keep theirs); starve = 1
+ * (needs wait_ns > 0) makes each of these kernels' producer of its first
+ * operand issue no copy, so its consumers' waits run out: the kernel frees its
+ * tensor memory, returns, and the next synchronising call of the handle reports
+ * DSANLS_ETIMEOUT (an iteration graph keeps what was set when it was captured).
+ * EINVAL for starve outside {0, 1} or starve without a limit;
+ * ECUDA if the device symbols cannot be written.  Synchronous. */
 int dsanls_debug_fail_alloc_after(int64_t n);
 int dsanls_debug_tc_wait(uint64_t wait_ns, int32_t starve);
 /* Index checks of the debug build: a library compiled with -DDSANLS_BOUNDS

@@ -176,8 +176,8 @@ def debug_fail_alloc_after(n):
 
 def debug_tc_wait(wait_ns=0, starve=False):
     """Test switch of the tensor-core kernels' bounded waits on the current
-    device: a limit of wait_ns (0: the default 2 s) and, with starve, a GEMM
-    producer that issues no copy so the waits run out."""
+    device: a limit of wait_ns (0: the default 2 s) and, with starve, producers
+    that issue no copy so the waits run out."""
     _check(lib().dsanls_debug_tc_wait(int(wait_ns), int(bool(starve))), "debug_tc_wait")
 
 

@@ -76,7 +76,6 @@ constexpr int RT_MAX_M = 6, RT_BST = 2;
 constexpr int RT_BSTAGE = RT_PARTS * RT_BN * 128;    // V's parts of a tile and K block
 constexpr int RT_CARRY = 16;                         // tiles between carries into FP64
 constexpr int64_t RT_GRID_SUMS = 512;                // doubles of `work` before k_parts_grid's sums
-constexpr unsigned long long RT_WAIT_NS = 2000000000ull;
 
 struct __align__(16) RtTail {
     uint64_t mfull[RT_MAX_M], mempty[RT_MAX_M];
@@ -97,19 +96,6 @@ struct RtCfg {
     static constexpr size_t SMEM = 1024 + ABYTES + RT_BST * RT_BSTAGE + MST * RT_CHUNK_BYTES + sizeof(RtTail);
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
-
-DSANLS_DEV bool rt_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer_ns();
-    while (!mbar_try_wait(bar, parity)) {
-        if (*abort) return false;
-        if (globaltimer_ns() - t0 > RT_WAIT_NS) {
-            *abort = 1;
-            return false;
-        }
-    }
-    return true;
-}
 
 // Two binary32 operations, rounded to nearest, in one instruction.
 DSANLS_DEV uint64_t rt_pair(float a, float b) {
@@ -157,7 +143,7 @@ template <int KB>
 __global__ void __launch_bounds__(RT_THREADS, 1)
     k_residual_tc(const __grid_constant__ CUtensorMap map_m, const __grid_constant__ CUtensorMap map_u,
                   const __grid_constant__ CUtensorMap map_v, int64_t m, int64_t n, int k, int64_t urows, int64_t vrows,
-                  const double *__restrict__ mm, double *__restrict__ part, int *__restrict__ err) {
+                  const double *__restrict__ mm, double *__restrict__ part, int *__restrict__ err, WaitSwitch wait) {
     using Cfg = RtCfg<KB>;
     constexpr int MST = Cfg::MST, APART = RT_BM * 128, BPART = RT_BN * 128;
     extern __shared__ __align__(1024) uint8_t rt_raw[];
@@ -208,7 +194,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
         const uint64_t scale = rt_pair(sc, sc);
         for (int i = 0; i < nt; ++i) {
             const int c = 2 * i + (cg >> 1), slot = c % MST, buf = i & 1;
-            bool ok = rt_wait(&tail->mfull[slot], (c / MST) & 1, abort);
+            bool ok = role_wait(&tail->mfull[slot], (c / MST) & 1, abort, wait.ns);
             if (!__all_sync(0xffffffffu, ok)) break;
             const float4 *row = reinterpret_cast<const float4 *>(mp + slot * RT_CHUNK_BYTES) + r * (RT_CHUNK / 4);
             float4 v[4];
@@ -218,7 +204,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
                 __syncwarp();  // 1.79 ms, 2.44 with the arrival below; k = 64, three tiles, 1.30 and 1.23)
                 if (lane == 0) mbar_arrive(&tail->mempty[slot]);
             }
-            ok = rt_wait(&tail->dfull[buf], (i >> 1) & 1, abort);
+            ok = role_wait(&tail->dfull[buf], (i >> 1) & 1, abort, wait.ns);
             if (!__all_sync(0xffffffffu, ok)) break;
             fence_after();
             uint32_t d[16], d1[16], d2[16], d3[16];
@@ -268,16 +254,16 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
                 const int buf = i & 1;
                 if (row != rt) {
                     if (na > 0) mma_commit(&tail->aempty);
-                    if (!rt_wait(&tail->afull, na & 1, abort)) break;
+                    if (!role_wait(&tail->afull, na & 1, abort, wait.ns)) break;
                     rt = row;
                     ++na;
                 }
-                if (i >= 2 && !rt_wait(&tail->dempty[buf], ((i >> 1) - 1) & 1, abort)) break;
+                if (i >= 2 && !role_wait(&tail->dempty[buf], ((i >> 1) - 1) & 1, abort, wait.ns)) break;
                 const uint32_t d = tmem + buf * RT_DSET;
                 bool ok = true;
                 for (int kb = 0; kb < KB; ++kb) {
                     const int b = i * KB + kb, sb = b % RT_BST;
-                    ok = rt_wait(&tail->bfull[sb], (b / RT_BST) & 1, abort);
+                    ok = role_wait(&tail->bfull[sb], (b / RT_BST) & 1, abort, wait.ns);
                     if (!ok) break;
                     fence_after();
                     const int nks = min(4, steps - 4 * kb);
@@ -297,15 +283,15 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
             }
             // every product this thread issued has retired before the tensor memory is freed
             mma_commit(&tail->fin);
-            mbar_wait(&tail->fin, 0, RT_WAIT_NS);
+            mbar_wait(&tail->fin, 0, wait.ns);
         }
     } else if (warp == RT_EW + 1) {
-        if (lane == 0) {
+        if (lane == 0 && !wait.starve) {
             // ---- tma M ----
             int issued = 0;
             for (int c = 0; c < 2 * nt; ++c) {
                 const int slot = c % MST;
-                if (c >= MST && !rt_wait(&tail->mempty[slot], ((c / MST) - 1) & 1, abort)) break;
+                if (c >= MST && !role_wait(&tail->mempty[slot], ((c / MST) - 1) & 1, abort, wait.ns)) break;
                 const int64_t t = t0 + (c >> 1);
                 mbar_expect_tx(&tail->mfull[slot], RT_CHUNK_BYTES);
                 tma_load_2d(mp + slot * RT_CHUNK_BYTES, &map_m, (int)((t % ntn) * RT_BN + (c & 1) * RT_CHUNK),
@@ -314,7 +300,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
             }
             if (*abort)  // nobody may be waiting for the last copies any more
                 for (int c = max(0, issued - MST); c < issued; ++c)
-                    mbar_wait(&tail->mfull[c % MST], (c / MST) & 1, RT_WAIT_NS);
+                    mbar_wait(&tail->mfull[c % MST], (c / MST) & 1, wait.ns);
         }
     } else if (lane == 0) {
         // ---- tma U, V (part p of K block kb: rows p urows + i, columns 64 kb ..) ----
@@ -324,7 +310,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
         for (int i = 0; ok && i < nt; ++i) {
             const int64_t row = (t0 + i) / ntn;
             if (row != rt) {
-                if (na > 0 && !rt_wait(&tail->aempty, (na - 1) & 1, abort)) break;
+                if (na > 0 && !role_wait(&tail->aempty, (na - 1) & 1, abort, wait.ns)) break;
                 mbar_expect_tx(&tail->afull, Cfg::ABYTES);
                 for (int x = 0; x < RT_PARTS * KB; ++x)
                     tma_load_2d(ap + x * APART, &map_u, (x / RT_PARTS) * 64,
@@ -334,7 +320,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
             }
             for (int kb = 0; kb < KB; ++kb) {
                 const int b = i * KB + kb, sb = b % RT_BST;
-                ok = b < RT_BST || rt_wait(&tail->bempty[sb], ((b / RT_BST) - 1) & 1, abort);
+                ok = b < RT_BST || role_wait(&tail->bempty[sb], ((b / RT_BST) - 1) & 1, abort, wait.ns);
                 if (!ok) break;
                 mbar_expect_tx(&tail->bfull[sb], RT_BSTAGE);
                 for (int p = 0; p < RT_PARTS; ++p)
@@ -344,9 +330,9 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
             }
         }
         if (*abort) {
-            if (na > 0) mbar_wait(&tail->afull, (na - 1) & 1, RT_WAIT_NS);
+            if (na > 0) mbar_wait(&tail->afull, (na - 1) & 1, wait.ns);
             for (int b = max(0, issued - RT_BST); b < issued; ++b)
-                mbar_wait(&tail->bfull[b % RT_BST], (b / RT_BST) & 1, RT_WAIT_NS);
+                mbar_wait(&tail->bfull[b % RT_BST], (b / RT_BST) & 1, wait.ns);
         }
     }
     double v = sum + rt_total(hi, lo);
@@ -493,7 +479,7 @@ template <int KB>
 void residual_launch(const CUtensorMap &mm_map, const CUtensorMap &mu, const CUtensorMap &mv, int64_t m, int64_t n, int k,
                      const double *mm, double *work, int grid, int *err, cudaStream_t s) {
     k_residual_tc<KB><<<grid, RT_THREADS, RtCfg<KB>::SMEM, s>>>(mm_map, mu, mv, m, n, k, pad_rows(m, RT_BM),
-                                                                pad_rows(n, RT_BN), mm, work, err);
+                                                                pad_rows(n, RT_BN), mm, work, err, wait_switch());
     DSANLS_LAUNCH_CHECK();
 }
 
@@ -552,5 +538,6 @@ void prime_residual_attributes(int max_smem) {
     allow_max_dynamic_smem(k_residual_tc<1>, max_smem);
     allow_max_dynamic_smem(k_residual_tc<2>, max_smem);
 }
+
 
 }  // namespace dsanls

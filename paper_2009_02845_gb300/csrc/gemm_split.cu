@@ -66,7 +66,6 @@ constexpr int SG_RK = 32;     // K of one step
 constexpr int SG_RAW_BYTES = SG_BM * SG_RK * 4;
 constexpr int SG_MAX_RAW = 8, SG_MAX_BST = 3, SG_MAX_AST = 4;
 constexpr int SG_ACOLS = 3 * SG_RK / 2;  // tensor-memory columns of the parts of one step of A
-constexpr unsigned long long SG_WAIT_NS = 2000000000ull;
 
 template <int BN>
 struct SgCfg {
@@ -101,22 +100,8 @@ constexpr size_t sg_smem() {
     return 1024 + SgCfg<BN>::BST * (size_t)SgCfg<BN>::BBYTES + SgCfg<BN>::RAW * SG_RAW_BYTES + sizeof(SgTail);
 }
 
-// bounded wait that also gives up once another role has given up
-DSANLS_DEV bool sg_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer_ns();
-    while (!mbar_try_wait(bar, parity)) {
-        if (*abort) return false;
-        if (globaltimer_ns() - t0 > SG_WAIT_NS) {
-            *abort = 1;
-            return false;
-        }
-    }
-    return true;
-}
-
 // wait (bounded) for the gate's count of ready steps to exceed st; the count, or <= st when giving up
-DSANLS_DEV int sg_poll(const int *count, int st, volatile int *abort) {
+DSANLS_DEV int sg_poll(const int *count, int st, volatile int *abort, unsigned long long limit) {
     int n = 0;
     unsigned long long t0 = 0;
     for (int spin = 1;; ++spin) {
@@ -125,7 +110,7 @@ DSANLS_DEV int sg_poll(const int *count, int st, volatile int *abort) {
         if ((spin & 255) == 0) {
             const unsigned long long t = globaltimer_ns();
             if (t0 == 0) t0 = t;
-            if (t - t0 > SG_WAIT_NS) {
+            if (t - t0 > limit) {
                 *abort = 1;
                 return n;
             }
@@ -180,7 +165,7 @@ template <int BN, bool AK, int NPB>
 __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
     k_split_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int64_t M,
                  int64_t N, int64_t K, const float *__restrict__ A, int64_t lda, const int32_t *__restrict__ gather,
-                 int tma, int avec, float *__restrict__ C, int64_t ldm, int64_t ldn, float alpha, int kb_per_split,
+                 int tma, int avec, WaitSwitch wait, float *__restrict__ C, int64_t ldm, int64_t ldn, float alpha, int kb_per_split,
                  int64_t c_split_stride, int *__restrict__ err) {
     using Cfg = SgCfg<BN>;
     constexpr int CW = Cfg::CW, AW = Cfg::AW, NSET = Cfg::NSET, FLUSH = Cfg::FLUSH, RAW = Cfg::RAW;
@@ -279,15 +264,15 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
             sg_copies_arrive(&tail->rfull[st % RAW]);
         };
         int next = -1;  // row_index of step st + RAW
-        if (!tma) {
+        if (!tma && !wait.starve) {
             for (int st = gr; st < RAW; st += 2)
                 if (st < nst) copy_step(st, row_index(st));
             next = row_index(RAW + gr);
         }
         for (int st = gr; st < nst; st += 2) {
             const int slot = st % RAW, sa = st % AST;
-            bool ok = sg_wait(&tail->rfull[slot], (st / RAW) & 1, abort);
-            if (ok && st >= AST) ok = sg_wait(&tail->aempty[sa], ((st / AST) - 1) & 1, abort);
+            bool ok = role_wait(&tail->rfull[slot], (st / RAW) & 1, abort, wait.ns);
+            if (ok && st >= AST) ok = role_wait(&tail->aempty[sa], ((st / AST) - 1) & 1, abort, wait.ns);
             if (!__all_sync(0xffffffffu, ok)) break;
             fence_after();
 #pragma unroll
@@ -308,7 +293,7 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
                 mbar_arrive(&tail->rempty[slot]);
             }
             if (!tma && st + RAW < nst) {  // the slot is free once the group has read it
-                const bool free = sg_wait(&tail->rempty[slot], (st / RAW) & 1, abort);
+                const bool free = role_wait(&tail->rempty[slot], (st / RAW) & 1, abort, wait.ns);
                 if (!__all_sync(0xffffffffu, free)) break;
                 copy_step(st + RAW, next);
                 next = row_index(st + RAW + 2);
@@ -327,7 +312,7 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
         bool ok = true;
         for (int iv = 0; iv < niv; ++iv) {
             const int buf = iv % NSET;
-            ok = __all_sync(0xffffffffu, sg_wait(&tail->dfull[buf], (iv / NSET) & 1, abort));
+            ok = __all_sync(0xffffffffu, role_wait(&tail->dfull[buf], (iv / NSET) & 1, abort, wait.ns));
             if (!ok) break;
             fence_after();
 #pragma unroll
@@ -373,7 +358,7 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
             for (int st = 0; st < nst; ++st) {
                 const int kb = st >> 1, sb = kb % BST, sa = st % AST, iv = kb / FLUSH, buf = iv % NSET;
                 const bool first = st % (2 * FLUSH) == 0;
-                if (ready <= st) ready = sg_poll(&tail->ready, st, abort);
+                if (ready <= st) ready = sg_poll(&tail->ready, st, abort, wait.ns);
                 if (ready <= st) break;
                 fence_after();
                 const uint32_t ah = tmem + Cfg::ACOL + sa * SG_ACOLS, am = ah + SG_RK / 2, al = am + SG_RK / 2;
@@ -405,7 +390,7 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
             }
             // every product this thread issued has retired before the tensor memory is freed
             mma_commit(&tail->fin);
-            mbar_wait(&tail->fin, 0, SG_WAIT_NS);
+            mbar_wait(&tail->fin, 0, wait.ns);
         }
     } else if (warp == CW + AW + 3) {
         if (lane == 0) {
@@ -413,10 +398,10 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
             for (int st = 0; st < nst; ++st) {
                 const int kb = st >> 1, iv = kb / FLUSH;
                 if (st % (2 * FLUSH) == 0 && iv >= NSET &&
-                    !sg_wait(&tail->dempty[iv % NSET], ((iv / NSET) - 1) & 1, abort))
+                    !role_wait(&tail->dempty[iv % NSET], ((iv / NSET) - 1) & 1, abort, wait.ns))
                     break;
-                if ((st & 1) == 0 && !sg_wait(&tail->bfull[kb % BST], (kb / BST) & 1, abort)) break;
-                if (!sg_wait(&tail->afull[st % AST], (st / AST) & 1, abort)) break;
+                if ((st & 1) == 0 && !role_wait(&tail->bfull[kb % BST], (kb / BST) & 1, abort, wait.ns)) break;
+                if (!role_wait(&tail->afull[st % AST], (st / AST) & 1, abort, wait.ns)) break;
                 fence_after();
                 fence_before();
                 asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tail->ready)), "r"(st + 1)
@@ -424,12 +409,12 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
             }
         }
     } else if (warp == CW + AW + 1) {
-        if (tma && lane == 0) {
+        if (tma && lane == 0 && !wait.starve) {
             // ---- tma A ----
             int issued = 0;
             for (int st = 0; st < nst; ++st) {
                 const int slot = st % RAW;
-                if (st >= RAW && !sg_wait(&tail->rempty[slot], ((st / RAW) - 1) & 1, abort)) break;
+                if (st >= RAW && !role_wait(&tail->rempty[slot], ((st / RAW) - 1) & 1, abort, wait.ns)) break;
                 float *dst = raw + slot * (SG_RAW_BYTES / 4);
                 const int k0 = (int)(kbeg + st * SG_RK);
                 mbar_expect_tx(&tail->rfull[slot], SG_RAW_BYTES);
@@ -441,14 +426,14 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
             }
             if (*abort)  // nobody may be waiting for the last copies any more
                 for (int st = max(0, issued - RAW); st < issued; ++st)
-                    mbar_wait(&tail->rfull[st % RAW], (st / RAW) & 1, SG_WAIT_NS);
+                    mbar_wait(&tail->rfull[st % RAW], (st / RAW) & 1, wait.ns);
         }
     } else if (lane == 0) {
         // ---- tma B ----
         int issued = 0;
         for (int kb = 0; kb < nkb; ++kb) {
             const int s = kb % BST;
-            if (kb >= BST && !sg_wait(&tail->bempty[s], ((kb / BST) - 1) & 1, abort)) break;
+            if (kb >= BST && !role_wait(&tail->bempty[s], ((kb / BST) - 1) & 1, abort, wait.ns)) break;
             uint8_t *dst = bst + s * Cfg::BBYTES;
             mbar_expect_tx(&tail->bfull[s], NPB * BPART);
             for (int p = 0; p < NPB; ++p)
@@ -457,7 +442,7 @@ __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
         }
         if (*abort)
             for (int kb = max(0, issued - BST); kb < issued; ++kb)
-                mbar_wait(&tail->bfull[kb % BST], (kb / BST) & 1, SG_WAIT_NS);
+                mbar_wait(&tail->bfull[kb % BST], (kb / BST) & 1, wait.ns);
     }
     fence_before();
     __syncthreads();
@@ -514,7 +499,7 @@ void sg_launch(const SplitGemm &g, float *dst, int64_t ldm, int64_t ldn, const S
     else if (tma)
         encode_f32_map(&ma, g.A, g.K, g.M, g.lda, SG_BM, SG_RK, false);
     const auto kernel = g.a_kcontig ? k_split_gemm<BN, true, NPB> : k_split_gemm<BN, false, NPB>;
-    kernel<<<grid, SgCfg<BN>::THREADS, sg_smem<BN>(), s>>>(ma, mb, g.M, g.N, g.K, g.A, g.lda, g.gather, tma, avec, dst,
+    kernel<<<grid, SgCfg<BN>::THREADS, sg_smem<BN>(), s>>>(ma, mb, g.M, g.N, g.K, g.A, g.lda, g.gather, tma, avec, wait_switch(), dst,
                                                            ldm, ldn, g.alpha, p.kb_per_split, g.M * g.N, err);
     DSANLS_LAUNCH_CHECK();
 }
@@ -610,5 +595,6 @@ void prime_split_gemm_attributes(int max_smem) {
     prime_sg<64, 3>(max_smem);
     prime_sg<128, 3>(max_smem);
 }
+
 
 }  // namespace dsanls

@@ -27,6 +27,7 @@
 #include <cuda_fp8.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -52,9 +53,10 @@ constexpr int kMaxSplits = 32;                         // split-K slices of the 
 }  // namespace
 
 // Test switch of the bounded waits (dsanls_debug_tc_wait): g_wait_ns > 0
-// replaces the 2 s limit of every tensor-core kernel's waits, and g_starve = 1
-// makes the TMA producer of k_tc_gemm issue no copy at all, so the waits on
-// its copies run out (nothing is in flight) and the kernel reports a timeout.
+// replaces the 2 s limit of this file's waits, and g_starve = 1 makes the TMA
+// producer of k_tc_gemm issue no copy at all, so the waits on its copies run out
+// (nothing is in flight) and the kernel reports a timeout.  The other tensor-core
+// kernels get the same two as an argument (wait_switch).
 __device__ unsigned long long g_wait_ns = 0;
 __device__ int g_starve = 0;
 
@@ -942,9 +944,23 @@ void launch_tc_skinny_split3(const __nv_bfloat16 *const X3[3], const __nv_bfloat
     launch_split_reduce(part, rows * k, p.splits, rows, k, k, R, k, s);
 }
 
+namespace {
+std::atomic<unsigned long long> g_launch_wait_ns{0};
+std::atomic<int> g_launch_starve{0};
+}  // namespace
+
+WaitSwitch wait_switch() {
+    WaitSwitch w;
+    if (const unsigned long long ns = g_launch_wait_ns.load()) w.ns = ns;
+    w.starve = g_launch_starve.load();
+    return w;
+}
+
 void set_tc_wait_debug(unsigned long long wait_ns, int starve) {
     DSANLS_CUDA(cudaMemcpyToSymbol(g_wait_ns, &wait_ns, sizeof(wait_ns)));
     DSANLS_CUDA(cudaMemcpyToSymbol(g_starve, &starve, sizeof(starve)));
+    g_launch_wait_ns = wait_ns;
+    g_launch_starve = starve;
 }
 
 void prime_tc_attributes(int max_smem) {

@@ -114,9 +114,17 @@ void launch_update_tc_subcsr(ZT *Z, const float *R, const SubCsr &sc, const ZT *
 // failed index checks of the debug build in tc_gemm.cu (see bounds_report_subcsr)
 void bounds_report_tc(int reset, int64_t out[3]);
 void prime_tc_attributes(int max_smem);
-// Test switch of the bounded waits on the current device: wait_ns > 0 replaces the
-// 2 s limit (0 restores it); starve = 1 makes the producer of the tensor-core GEMM
-// issue no copy, so its consumers' waits run out and report DSANLS_ETIMEOUT.
+// Test switch of the bounded waits: wait_ns > 0 replaces the 2 s limit (0 restores it);
+// starve = 1 makes the producer of a kernel's first operand issue no copy, so its consumers'
+// waits run out and report DSANLS_ETIMEOUT.  k_tc_gemm reads it on the current device; the
+// other kernels get it with their launch (a captured one keeps what was set then), for the
+// first read of a device variable costs a kernel that waits right after its launch 0.4 us,
+// 2 % of a small FP32 product.
+struct WaitSwitch {
+    unsigned long long ns = 2000000000ull;
+    int starve = 0;
+};
+WaitSwitch wait_switch();
 void set_tc_wait_debug(unsigned long long wait_ns, int starve);
 
 }  // namespace dsanls

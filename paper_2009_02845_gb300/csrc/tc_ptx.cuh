@@ -56,6 +56,20 @@ DSANLS_DEV bool mbar_wait(uint64_t *bar, uint32_t parity, unsigned long long lim
     return true;
 }
 
+// Wait of one role of a kernel: gives up at the limit or once another role has (*abort).
+DSANLS_DEV bool role_wait(uint64_t *bar, uint32_t parity, volatile int *abort, unsigned long long limit) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const unsigned long long t0 = globaltimer_ns();
+    while (!mbar_try_wait(bar, parity)) {
+        if (*abort) return false;
+        if (globaltimer_ns() - t0 > limit) {
+            *abort = 1;
+            return false;
+        }
+    }
+    return true;
+}
+
 // 2-D tiled TMA load of the box at (x, y) (x: innermost, elements) of the tensor
 // map into shared memory; its bytes complete the transaction count of `bar`.
 // The map is in kernel-parameter, constant or global memory.

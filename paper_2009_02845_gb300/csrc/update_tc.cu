@@ -61,8 +61,6 @@ template <typename ZT>
 __host__ __device__ constexpr int upd_groups() {
     return sizeof(ZT) == 2 ? 3 : 2;
 }
-constexpr unsigned long long UPD_WAIT_NS = 2000000000ull;
-constexpr long long UPD_WAIT_CLK = 4000000000ll;
 
 struct __align__(8) UpdTail {
     uint64_t zfull[UPD_MAX_NZ], zempty[UPD_MAX_NZ];  // pieces of Z
@@ -72,19 +70,6 @@ struct __align__(8) UpdTail {
     uint32_t tmem_base;
     int abort;
 };
-
-DSANLS_DEV bool upd_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
-        if (*abort) return false;
-        if (clock64() - t0 > UPD_WAIT_CLK) {
-            *abort = 1;
-            return false;
-        }
-    }
-    return true;
-}
 
 DSANLS_DEV float upd_project(float v, float bound, int *flag) {
     if (!(fabsf(v) <= 3.402823466e38f)) {  // NaN or Inf
@@ -242,7 +227,7 @@ template <typename ZT, bool SPR, bool VEC>
 __global__ void __launch_bounds__(UPD_THREADS)
     k_update_tc(ZT *__restrict__ Z, const float *__restrict__ R, int64_t rows, UpdShape sh,
                 const float *__restrict__ Gf, int kp, const double *__restrict__ scal, float bound,
-                int *__restrict__ flag, UpdSub<ZT> sub) {
+                int *__restrict__ flag, UpdSub<ZT> sub, WaitSwitch wait) {
     constexpr bool ZBF = sizeof(ZT) == 2;
     constexpr int UPD_STEP = UPD_STEPS / upd_groups<ZT>();  // warps of a step group
     constexpr int ZPARTS = ZBF ? 1 : 3;  // nonzero parts of the split of z
@@ -264,15 +249,15 @@ __global__ void __launch_bounds__(UPD_THREADS)
     auto row_of = [&](int p) { return tile_of(p >> 2) * UPD_BM + 32 * (p & 3); };
     auto nrows = [&](int p) { return (int)min((int64_t)32, rows - row_of(p)); };
     auto zpiece = [&](int p) { return reinterpret_cast<ZT *>(zb + (p % sh.nz) * sh.zbytes); };
-    auto full_wait = [&](uint64_t *bars, int p, int n) { return upd_wait(&bars[p % n], (p / n) & 1, abort); };
+    auto full_wait = [&](uint64_t *bars, int p, int n) { return role_wait(&bars[p % n], (p / n) & 1, abort, wait.ns); };
     auto free_wait = [&](uint64_t *bars, int p, int n) {
-        return p < n || upd_wait(&bars[p % n], ((p / n) - 1) & 1, abort);
+        return p < n || role_wait(&bars[p % n], ((p / n) - 1) & 1, abort, wait.ns);
     };
 
     // R given: the first tile, when it is whole, is asked for while G is split, 1 us of the 7
     // that a CTA with one tile takes.  (SPR goes without: the same lines cost the code of its
     // step 11 % of 2e6 rows in bf16, 484 -> 530 us.)
-    const bool early = !SPR && sh.bulk && ((int64_t)blockIdx.x + 1) * UPD_BM <= rows;
+    const bool early = !SPR && sh.bulk && ((int64_t)blockIdx.x + 1) * UPD_BM <= rows && !wait.starve;
     if (warp == w_copy) {
         if (lane == 0) {
             for (int i = 0; i < sh.nz; ++i) {
@@ -484,11 +469,11 @@ __global__ void __launch_bounds__(UPD_THREADS)
         }
         // every product of this warp has retired before the tensor memory is freed
         upd_commit(&tail->fin);
-        mbar_wait(&tail->fin, 0, UPD_WAIT_NS);
+        mbar_wait(&tail->fin, 0, wait.ns);
     } else if (warp == w_copy) {
         // ---- copy ----
         int issued = early ? 4 : 0;
-        for (int p = issued; p < 4 * nt; ++p) {
+        for (int p = issued; p < 4 * nt && !wait.starve; ++p) {
             const int nr = max(0, nrows(p));
             const uint32_t bytes = (uint32_t)(nr * k * (int)sizeof(ZT));
             if (!__all_sync(0xffffffffu, free_wait(tail->zempty, p, sh.nz))) break;
@@ -509,7 +494,7 @@ __global__ void __launch_bounds__(UPD_THREADS)
         }
         if (*abort && lane == 0)  // nobody may be waiting for the last copies any more
             for (int p = max(0, issued - sh.nz); p < issued; ++p)
-                mbar_wait(&tail->zfull[p % sh.nz], (p / sh.nz) & 1, UPD_WAIT_NS);
+                mbar_wait(&tail->zfull[p % sh.nz], (p / sh.nz) & 1, wait.ns);
     }
     fence_before();
     __syncthreads();
@@ -545,7 +530,7 @@ void launch_update_tc_any(ZT *Z, const float *R, int64_t rows, int k, const floa
     if (ntiles / grid >= (1ll << 28)) throw ArgError{"launch_update_tc: too many rows"};
     const size_t smem = fixed + sh.nz * (size_t)sh.zbytes;
     const auto kern = k % 4 == 0 ? k_update_tc<ZT, SPR, true> : k_update_tc<ZT, SPR, false>;
-    kern<<<(unsigned)grid, 32 * (UPD_SPLIT + sh.na * (UPD_STEPS / upd_groups<ZT>()) + 2), smem, s>>>(Z, R, rows, sh, Gf, kp, scal, bound, flag, sub);
+    kern<<<(unsigned)grid, 32 * (UPD_SPLIT + sh.na * (UPD_STEPS / upd_groups<ZT>()) + 2), smem, s>>>(Z, R, rows, sh, Gf, kp, scal, bound, flag, sub, wait_switch());
     DSANLS_LAUNCH_CHECK();
 }
 
@@ -597,5 +582,6 @@ void prime_update_attributes(int max_smem) {
     allow_max_dynamic_smem(k_update_tc<__nv_bfloat16, true, true>, max_smem);
     allow_max_dynamic_smem(k_update_tc<__nv_bfloat16, true, false>, max_smem);
 }
+
 
 }  // namespace dsanls
