@@ -406,7 +406,11 @@ int dsanls_mlp_get_params(dsanls_mlp_t m, float *theta);        /* host array of
 int dsanls_mlp_set_params(dsanls_mlp_t m, const float *theta);  /* host array of param_count */
 /* Device arrays: G (ngroups x k x k), mu (ngroups), group_off (ngroups + 1,
  * rows of group g are group_off[g] .. group_off[g+1]-1), b (rows x k, b = r + mu u).
- * x_out (rows x k) = the network's warm start in the original scale. */
+ * x_out (rows x k) = the network's warm start in the original scale.  Queued
+ * on `stream`.  If a bounded wait of its tensor-core products gives up, x_out
+ * is NaN throughout and the next dsanls_mlp_get_params or dsanls_mlp_set_params
+ * (whose own work is done all the same) returns DSANLS_ETIMEOUT, once; training
+ * has no such wait and does not report it. */
 int dsanls_mlp_predict(dsanls_mlp_t m, const float *G, const float *mu, const int64_t *group_off, int32_t ngroups,
                        const float *b, int64_t rows, float *x_out, void *stream);
 /* Loss 1/2 mean ||y - y*||^2 against the normalised exact minimisers

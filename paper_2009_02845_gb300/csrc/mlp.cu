@@ -80,10 +80,11 @@ __global__ void k_adam_round(float *__restrict__ theta, float *__restrict__ m, f
     put_parts(w3, i, q);
 }
 
-// per group: s_g and Gn_g
+// per group: s_g and Gn_g; the first kernel of a pass clears the word that the pass's products raise
 __global__ void k_norm_groups(const float *__restrict__ G, const float *__restrict__ mu, int k, int ngroups,
-                              float *__restrict__ Gn, float *__restrict__ s_out) {
+                              float *__restrict__ Gn, float *__restrict__ s_out, int *__restrict__ clear) {
     const int g = blockIdx.x;
+    if (clear && g == 0 && threadIdx.x == 0) *clear = 0;
     if (g >= ngroups) return;
     __shared__ float s_sh;
     const float *Gg = G + (int64_t)g * k * k;
@@ -350,7 +351,7 @@ void mlp_alloc(MlpState &st, int k, int h, int64_t max_rows, int max_groups) {
     al(st.bn, max_rows * k); al(st.beta, max_rows);
     al(st.z1, max_rows * h); al(st.h1, max_rows * h); al(st.z2, max_rows * h); al(st.h2, max_rows * h);
     al(st.o, max_rows * k); al(st.y, max_rows * k); al(st.dout, max_rows * k); al(st.rowloss, max_rows);
-    al(st.loss, 2);  // the loss, then the error word
+    al(st.loss, 2);  // the loss, then the error words
     st.err = reinterpret_cast<int *>(st.loss + 1);
     al(st.gf1, (int64_t)k * k); al(st.mu1, 1); al(st.off1, 2);
     al(st.W1g, h * split_parts_ld((int64_t)k * k)); al(st.W1b, h * split_parts_ld(k)); al(st.W2, h * split_parts_ld(h));
@@ -424,7 +425,7 @@ void mlp_forward(MlpState &st, const float *G, const float *mu, const int64_t *o
     const int64_t kk = (int64_t)k * k;
     const MlpOffsets O = mlp_offsets(k, h);
     const float *W = st.wq;
-    k_norm_groups<<<ngroups, 128, 0, s>>>(G, mu, k, ngroups, st.Gn, st.s);
+    k_norm_groups<<<ngroups, 128, 0, s>>>(G, mu, k, ngroups, st.Gn, st.s, err == st.err ? err : nullptr);
     DSANLS_LAUNCH_CHECK();
     if (training)
         chain(ngroups, h, kk, st.Gn, kk, true, W + O.W1g, kk, true, st.zg, h, s);
@@ -527,15 +528,19 @@ void mlp_init(MlpState &st, uint64_t seed, cudaStream_t s) {
 }
 
 __global__ void k_unscale(const float *__restrict__ y, const float *__restrict__ s_g, const float *__restrict__ beta,
-                          const int64_t *__restrict__ off, int ngroups, int64_t rows, int k, float *__restrict__ x) {
+                          const int64_t *__restrict__ off, int ngroups, int64_t rows, int k, int *__restrict__ err,
+                          float *__restrict__ x) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * k) return;
     const int64_t r = idx / k;
-    x[idx] = y[idx] * beta[r] / s_g[group_of(off, ngroups, r)];
+    // a product gave up: no number that could pass for a prediction, and the handle is told
+    const bool failed = err[0] != 0;
+    if (failed && idx == 0) err[1] = 1;
+    x[idx] = failed ? __int_as_float(0x7fc00000) : y[idx] * beta[r] / s_g[group_of(off, ngroups, r)];
 }
 
 void mlp_unscale(MlpState &st, const int64_t *off, int ngroups, int64_t rows, float *x_out, cudaStream_t s) {
-    k_unscale<<<nblk(rows * st.k), 256, 0, s>>>(st.y, st.s, st.beta, off, ngroups, rows, st.k, x_out);
+    k_unscale<<<nblk(rows * st.k), 256, 0, s>>>(st.y, st.s, st.beta, off, ngroups, rows, st.k, st.err, x_out);
     DSANLS_LAUNCH_CHECK();
 }
 

@@ -24,7 +24,9 @@ struct MlpState {
     float *z1 = nullptr, *h1 = nullptr, *z2 = nullptr, *h2 = nullptr;
     float *o = nullptr, *y = nullptr, *dout = nullptr;
     double *rowloss = nullptr, *loss = nullptr;
-    int *err = nullptr;  // raised when a product's bounded wait gives up (after the loss)
+    // [0] raised when a product of the running prediction gives up its bounded wait, [1] left by
+    // such a prediction until a synchronising call has reported it (both behind the loss)
+    int *err = nullptr;
     // the rounded weights as second operands of prediction's products
     __nv_bfloat16 *W1g = nullptr, *W1b = nullptr, *W2 = nullptr, *W3 = nullptr;
     float *part = nullptr;  // split-K partials
@@ -42,7 +44,7 @@ void mlp_alloc(MlpState &st, int k, int h, int64_t max_rows, int max_groups);
 void mlp_free(MlpState &st);
 void mlp_quantise(MlpState &st, cudaStream_t s);
 void mlp_forward(MlpState &st, const float *G, const float *mu, const int64_t *off, int ngroups, const float *b,
-                 int64_t rows, bool training, int *err, cudaStream_t s);
+                 int64_t rows, bool training, int *err, cudaStream_t s);  // (training raises no *err)
 // buffers and streams of the backward pass (at the first training step)
 void mlp_reserve_training(MlpState &st);
 // after a training forward pass: loss and gradient against y* = x* s_g / beta_r
@@ -58,7 +60,8 @@ void mlp_harvest(const float *Z, const float *R, const float *Gf, int kp, const 
                  int iters, float *b_out, float *x_out, cudaStream_t s);
 // theta ~ U(-sqrt(3/fan_in), sqrt(3/fan_in)) from Philox stream 0x20 keyed by seed; biases 0.
 void mlp_init(MlpState &st, uint64_t seed, cudaStream_t s);
-// x0 = y beta_r / s_g (the warm start in the original scale) after mlp_forward.
+// x0 = y beta_r / s_g (the warm start in the original scale) after mlp_forward with st.err; NaN
+// when that was raised.
 void mlp_unscale(MlpState &st, const int64_t *off, int ngroups, int64_t rows, float *x_out, cudaStream_t s);
 
 }  // namespace dsanls

@@ -2,7 +2,6 @@
 // prediction and one training step (forward, backward, Adam).
 #include <cuda_runtime.h>
 
-#include <cstring>
 #include <new>
 #include <string>
 
@@ -42,6 +41,16 @@ int check_batch(const dsanls_mlp_ctx *m, const float *G, const float *mu, const 
         return DSANLS_EINVAL;
     }
     return DSANLS_OK;
+}
+
+// after a synchronisation: the timeout that a prediction since the last report left, if any
+int pending_prediction(dsanls_mlp_ctx *m) {
+    int failed = 0;
+    DSANLS_CUDA(cudaMemcpy(&failed, m->st.err + 1, sizeof failed, cudaMemcpyDeviceToHost));
+    if (!failed) return DSANLS_OK;
+    DSANLS_CUDA(cudaMemset(m->st.err + 1, 0, sizeof(int)));
+    record_handleless_error("a prediction gave up a bounded device wait (its x is NaN)");
+    return DSANLS_ETIMEOUT;
 }
 
 }  // namespace
@@ -91,7 +100,7 @@ int dsanls_mlp_get_params(dsanls_mlp_t m, float *theta) {
         DSANLS_CUDA(cudaDeviceSynchronize());
         DSANLS_CUDA(cudaMemcpy(theta, m->st.theta, mlp_param_count(m->st.k, m->st.h) * sizeof(float),
                                cudaMemcpyDeviceToHost));
-        return DSANLS_OK;
+        return pending_prediction(m);
     });
 }
 
@@ -103,7 +112,7 @@ int dsanls_mlp_set_params(dsanls_mlp_t m, const float *theta) {
                                cudaMemcpyHostToDevice));
         mlp_quantise(m->st, m->own_stream);
         DSANLS_CUDA(cudaStreamSynchronize(m->own_stream));
-        return DSANLS_OK;
+        return pending_prediction(m);
     });
 }
 
@@ -131,23 +140,14 @@ int dsanls_mlp_train_step(dsanls_mlp_t m, const float *G, const float *mu, const
     return mguard([&]() {
         cudaStream_t s = (cudaStream_t)stream;
         mlp_reserve_training(m->st);
-        mlp_forward(m->st, G, mu, group_off, ngroups, b, rows, true, m->st.err, s);
+        mlp_forward(m->st, G, mu, group_off, ngroups, b, rows, true, nullptr, s);
         mlp_backward(m->st, group_off, ngroups, xstar, rows, s);
         if (grad)
             DSANLS_CUDA(cudaMemcpyAsync(grad, m->st.grad, mlp_param_count(m->st.k, m->st.h) * sizeof(float),
                                         cudaMemcpyDeviceToHost, s));
-        double out[2] = {0.0, 0.0};  // the loss and the error word behind it
-        DSANLS_CUDA(cudaMemcpyAsync(out, m->st.loss, sizeof out, cudaMemcpyDeviceToHost, s));
+        if (loss) DSANLS_CUDA(cudaMemcpyAsync(loss, m->st.loss, sizeof(double), cudaMemcpyDeviceToHost, s));
         if (lr > 0.0f) mlp_adam(m->st, lr, s);
         DSANLS_CUDA(cudaStreamSynchronize(s));
-        if (loss) *loss = out[0];
-        int err = 0;
-        std::memcpy(&err, &out[1], sizeof err);
-        if (err) {
-            DSANLS_CUDA(cudaMemset(m->st.err, 0, sizeof(int)));
-            record_handleless_error("a bounded device wait gave up (tensor-core pipeline)");
-            return DSANLS_ETIMEOUT;
-        }
         return DSANLS_OK;
     });
 }
