@@ -286,6 +286,7 @@ SplitNeed split_need(const dsanls_ctx *h) {
         const int64_t rows = side == 0 ? h->m : h->n, K = side == 0 ? h->n : h->m, k = h->k;
         const int64_t dd = side == 0 ? h->d : d_v_of(h);
         auto use = [&](int64_t M, int64_t N, int64_t L) {
+            if (!split_gemm_supported(M, N, L)) return;
             need.part = std::max(need.part, split_gemm_plan(M, N, L, SPLIT_GEMM_MAX_SPLITS).part_elems);
             need.parts = std::max(need.parts, 3 * N * split_parts_ld(L));
         };
@@ -447,7 +448,7 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
 
     // one of the FP32 form's products (c_trans: stored transposed, split products only)
     auto product = [&](const GemmArgs &g, bool c_trans = false) {
-        if (chained(h)) {
+        if (chained(h) || !split_gemm_supported(g.M, g.N, g.K)) {  // (A = X S of 7e8 columns)
             launch_sgemm(g, s);
             return;
         }

@@ -468,18 +468,20 @@ __global__ void k_parts_cols(const float *__restrict__ B, int64_t ldb, const int
                              int64_t K, int64_t ldk, __nv_bfloat16 *__restrict__ out) {
     __shared__ float tile[32][33];
     const int64_t k0 = (int64_t)blockIdx.x * 32;
-    const int64_t n0 = (int64_t)blockIdx.y * 32;
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int64_t k = k0 + y, n = n0 + threadIdx.x;
-        if (k < K && n < N) tile[y][threadIdx.x] = B[(gather ? (int64_t)gather[k] : k) * ldb + n];
-    }
-    __syncthreads();
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int64_t n = n0 + y, k = k0 + threadIdx.x;
-        if (k < K && n < N) {
-            __nv_bfloat16 *o = out + n * ldk + k;
-            split3_one(tile[threadIdx.x][y], o[0], o[N * ldk], o[2 * N * ldk]);
+    for (int64_t n0 = (int64_t)blockIdx.y * 32; n0 < N; n0 += (int64_t)gridDim.y * 32) {
+        for (int y = threadIdx.y; y < 32; y += blockDim.y) {
+            const int64_t k = k0 + y, n = n0 + threadIdx.x;
+            if (k < K && n < N) tile[y][threadIdx.x] = B[(gather ? (int64_t)gather[k] : k) * ldb + n];
         }
+        __syncthreads();
+        for (int y = threadIdx.y; y < 32; y += blockDim.y) {
+            const int64_t n = n0 + y, k = k0 + threadIdx.x;
+            if (k < K && n < N) {
+                __nv_bfloat16 *o = out + n * ldk + k;
+                split3_one(tile[threadIdx.x][y], o[0], o[N * ldk], o[2 * N * ldk]);
+            }
+        }
+        __syncthreads();  // the tile is free again
     }
 }
 
@@ -520,9 +522,8 @@ void launch_split_parts(const float *B, int64_t ldb, bool kcontig, const int32_t
                         (unsigned)std::min<int64_t>(ceil_div(K, tx), 64));
         k_parts_rows<<<grid, dim3(tx, ty), 0, s>>>(B, ldb, N, K, ldk, out);
     } else {
-        if (ceil_div(N, 32) > 65535) throw ArgError{"split parts: too many rows"};
-        k_parts_cols<<<dim3((unsigned)ceil_div(K, 32), (unsigned)ceil_div(N, 32)), dim3(32, 8), 0, s>>>(
-            B, ldb, gather, N, K, ldk, out);
+        const dim3 grid((unsigned)ceil_div(K, 32), (unsigned)std::min<int64_t>(ceil_div(N, 32), 65535));
+        k_parts_cols<<<grid, dim3(32, 8), 0, s>>>(B, ldb, gather, N, K, ldk, out);
     }
     DSANLS_LAUNCH_CHECK();
 }
@@ -554,12 +555,16 @@ SplitPlan split_gemm_plan(int64_t M, int64_t N, int64_t K, int max_splits) {
     return p;
 }
 
+bool split_gemm_supported(int64_t M, int64_t N, int64_t K) {
+    // coordinates of tensor maps (the three parts lie one below the other)
+    return M < (1ll << 31) && K < (1ll << 31) && 3 * N < (1ll << 31);
+}
+
 void launch_split_gemm(const SplitGemm &g, int *err, cudaStream_t s) {
     if (g.M <= 0 || g.N <= 0) return;
     if (g.K <= 0) throw ArgError{"split GEMM: K must be >= 1"};
     if (g.gather && g.a_kcontig) throw ArgError{"split GEMM: a gather needs K rows"};
-    if (g.M > (1ll << 31) - 1 || g.K > (1ll << 31) - 1 || 3 * g.N > (1ll << 31) - 1)
-        throw ArgError{"sizes too large"};
+    if (!split_gemm_supported(g.M, g.N, g.K)) throw ArgError{"sizes too large"};
     const SplitPlan p = split_gemm_plan(g.M, g.N, g.K, g.max_splits);
     float *dst = p.splits > 1 ? g.part : g.C;
     // partials keep C's orientation, so the reduction below is a plain sum of slices

@@ -118,6 +118,7 @@ struct SplitPlan {
     int64_t part_elems;
 };
 SplitPlan split_gemm_plan(int64_t M, int64_t N, int64_t K, int max_splits);
+bool split_gemm_supported(int64_t M, int64_t N, int64_t K);
 constexpr int SPLIT_GEMM_MAX_SPLITS = 64;
 void launch_split_gemm(const SplitGemm &g, int *err, cudaStream_t s);
 int64_t split_parts_ld(int64_t K);
