@@ -308,16 +308,37 @@ SplitNeed split_need(const dsanls_ctx *h) {
     return need;
 }
 
-// Sum of the d largest row lengths of a CSR row pointer (the most entries a
-// sampled set of d of its rows can hold).
-int64_t top_sum(const std::vector<int64_t> &ptr, int64_t d) {
+// Of a CSR row pointer: the sum of its d largest row lengths (the most entries a sampled set of
+// d of its rows can hold), and what its rows are expected to hold of a sample of the share f of
+// the columns.
+struct RowLengths {
+    int64_t top_sum = 0;
+    SubRows expected;
+};
+RowLengths row_lengths(const std::vector<int64_t> &ptr, int64_t d, double f) {
+    RowLengths r;
     std::vector<int64_t> len(ptr.size() > 0 ? ptr.size() - 1 : 0);
     for (size_t i = 0; i < len.size(); ++i) len[i] = ptr[i + 1] - ptr[i];
     d = std::min<int64_t>(d, (int64_t)len.size());
     std::nth_element(len.begin(), len.begin() + d, len.end(), std::greater<int64_t>());
-    int64_t s = 0;
-    for (int64_t i = 0; i < d; ++i) s += len[i];
-    return s;
+    r.expected.rows = (double)len.size();
+    r.expected.entries = len.empty() ? 0.0 : (double)ptr.back() * f;
+    const double cut = (double)SUB_LONG / f;
+    int64_t shortest = 0;  // of the d largest
+    auto add = [&](int64_t n) {
+        if ((double)n <= cut) return;
+        r.expected.long_rows += 1.0;
+        r.expected.long_entries += (double)n * f;
+        r.expected.longest = std::max(r.expected.longest, (double)n * f);
+    };
+    for (int64_t i = 0; i < d; ++i) {
+        r.top_sum += len[i];
+        shortest = i == 0 ? len[i] : std::min(shortest, len[i]);
+        add(len[i]);
+    }
+    if ((double)shortest > cut)  // (the others are no longer than that)
+        for (size_t i = (size_t)d; i < len.size(); ++i) add(len[i]);
+    return r;
 }
 
 // (Re)allocate the per-configuration workspaces.
@@ -392,8 +413,9 @@ void prepare(dsanls_ctx *h) {
     if (h->sketch == DSANLS_SKETCH_SUBSAMPLE && h->has_sparse) {
         // U-half: columns of M (rows of M^T), V-half: rows of M; room for the
         // longest possible sampled set of each side
-        h->sub[0].reserve(m, h->d, top_sum(h->h_trp, h->d), (double)h->nnz * h->d / ((double)m * n), h->stream());
-        h->sub[1].reserve(n, dv, top_sum(h->h_rp, dv), (double)h->nnz * dv / ((double)m * n), h->stream());
+        const RowLengths u = row_lengths(h->h_rp, dv, (double)h->d / n), v = row_lengths(h->h_trp, h->d, (double)dv / m);
+        h->sub[0].reserve(m, h->d, v.top_sum, u.expected, h->stream());
+        h->sub[1].reserve(n, dv, u.top_sum, v.expected, h->stream());
     } else {
         h->sub[0].release();
         h->sub[1].release();

@@ -207,8 +207,17 @@ constexpr int64_t SUB_LONG = 64;
 // Rows of more than this many are left to a warp each where one thread would walk them.
 constexpr int64_t SUB_MID = 16;
 // The entries are placed row by row and the rows sorted (instead of a radix sort over all
-// entries) when a row is expected to hold at most this many.
+// entries) when a row is expected to hold at most this many, and its long rows are few and short
+// enough (SubRows::place).
 constexpr double SUB_PLACE_AVG = 8.0;
+
+// The sampled entries that the rows are expected to hold.
+struct SubRows {
+    double rows = 0.0, entries = 0.0;             // all of them
+    double long_rows = 0.0, long_entries = 0.0;   // in rows of more than SUB_LONG
+    double longest = 0.0;
+    bool place() const;
+};
 
 struct SubCsr {
     int64_t rows = 0, cap = 0;
@@ -219,8 +228,7 @@ struct SubCsr {
     bool place = false;       // rows placed and sorted (else radix-sorted entries)
     int32_t *key[2] = {nullptr, nullptr}, *col[2] = {nullptr, nullptr};
     float *val[2] = {nullptr, nullptr};
-    // per_row: the entries a row is expected to hold
-    void reserve(int64_t rows, int dmax, int64_t cap, double per_row, cudaStream_t s);
+    void reserve(int64_t rows, int dmax, int64_t cap, const SubRows &expected, cudaStream_t s);
     int64_t warp_rows() const { return mids ? SUB_MID : SUB_LONG; }  // longer rows: launch_subcsr_long_rows
     void release();
 };

@@ -12,8 +12,8 @@
 //   3. the entries by row, in ascending e within a row: the CSR order of the row in X,
 //      which makes sums over a row deterministic and equal to a row-wise pass over X that
 //      skips the unsampled columns.  In one of two ways, by the expected number of sampled
-//      entries per row (SubCsr::reserve):
-//      few (<= SUB_PLACE_AVG): ptr = exclusive scan of cnt; every entry's e to the next free
+//      entries per row (SubRows::place):
+//      few (<= SUB_PLACE_AVG, and no row very long): ptr = exclusive scan of cnt; every entry's e to the next free
 //      place of its row, in whatever order the atomics fall; then each row is sorted by e --
 //      a row of <= SUB_MID entries by one thread, <= SUB_LONG by a warp, longer ones by a
 //      CTA's radix sort -- and its columns and values are fetched.  9 launches that each
@@ -550,9 +550,24 @@ static void sub_alloc(void **p, size_t bytes) {
     }
 }
 
-void SubCsr::reserve(int64_t rows_, int dmax_, int64_t cap_, double per_row, cudaStream_t s) {
+// A long row is one CTA's work, one after the other: beside the radix sort of all entries it
+// costs 10 us and 7.3 ns for each of its entries more (a row of 1,000 .. 65,000 sampled entries
+// among 20,000 .. 1e6 short ones; 100,000 rows of 66).  The radix sort costs 44 us and 62 ps for
+// each entry more than placing all of them.  So the longest row, and the long rows shared out
+// over 304 CTAs, may not take longer than that.  Build and long rows' sums, placed / radix: 1e6
+// rows of about one entry and one of 1,000 134 / 239 us, 8,000 249 / 302, 16,000 377 / 375,
+// 65,000 1,159 / 809, 1e6 16.1 / 9.0 ms; 60,000 rows and one of 4,000 171 / 198, 8,000 219 / 219,
+// 32,000 486 / 333; 1e6 rows, 2,000 of them of 3,500 1.09 / 1.25 ms, 20,000 of 300 1.51 / 1.38,
+// 100,000 of 66 4.78 / 2.64.
+bool SubRows::place() const {
+    const double spare = 44.0 + 62e-6 * entries;
+    return entries <= SUB_PLACE_AVG * rows && 7.3e-3 * longest <= spare &&
+           (10.0 * long_rows + 7.3e-3 * long_entries) / 304.0 <= spare;
+}
+
+void SubCsr::reserve(int64_t rows_, int dmax_, int64_t cap_, const SubRows &expected, cudaStream_t s) {
     if (rows_ > (1ll << 31) - 1) throw ArgError{"sub-CSR: more than 2^31 - 1 rows"};
-    const bool few = per_row <= SUB_PLACE_AVG;
+    const bool few = expected.place();
     if (rows == rows_ && dmax >= dmax_ && cap >= cap_ && off) {
         place = few && mids && cap < (1ll << 31);
         return;
