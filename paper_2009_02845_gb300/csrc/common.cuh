@@ -27,11 +27,17 @@ DSANLS_DEV Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t
                                  uint32_t k1) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint64_t p0 = (uint64_t)0xD2511F53u * c0, p1 = (uint64_t)0xCD9E8D57u * c2;  // one wide product each
-        c0 = (uint32_t)(p1 >> 32) ^ c1 ^ k0;
-        c1 = (uint32_t)p1;
-        c2 = (uint32_t)(p0 >> 32) ^ c3 ^ k1;
-        c3 = (uint32_t)p0;
+        // (as two 32-bit halves: one 64-bit product each made a Gaussian draw 8 % and a
+        // Rademacher one 19 % slower -- 65,536 x 2,048 in bf16 286 -> 309 us, 60,832 x 2,048 of
+        // signs 131 -> 157)
+        const uint32_t lo0 = 0xD2511F53u * c0;
+        const uint32_t hi0 = __umulhi(0xD2511F53u, c0);
+        const uint32_t lo1 = 0xCD9E8D57u * c2;
+        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2);
+        c0 = hi1 ^ c1 ^ k0;
+        c1 = lo1;
+        c2 = hi0 ^ c3 ^ k1;
+        c3 = lo0;
         k0 += 0x9E3779B9u;
         k1 += 0xBB67AE85u;
     }
@@ -53,10 +59,9 @@ DSANLS_DEV uint32_t word_of(const Philox4 &b, int r) {
 // pairs are about 250; the values leave at a third of the HBM rate), and integer-to-float
 // conversions run on the quarter-rate unit of the reciprocals.  So integers below 2^23 come to
 // binary32 as the fraction bits of a power of two, less that power: exact, like the
-// conversions they stand for.  65,536 x 2,048 normals:
-// bf16 S and S^T 301 -> 275 us, bf16 S^T 347 -> 311, bf16 and fp8 S^T 332 -> 302 (the
-// last two with one store a block in place of four and eight); 1,024 uneven instances 1.76
-// -> 1.50 ms.
+// conversions they stand for.  65,536 x 2,048 normals: bf16 S and S^T 300 -> 259 us, bf16 S^T
+// 345 -> 286, bf16 and fp8 S^T 338 -> 286 (the last two with one store a block in place of four
+// and eight); 1,024 uneven instances 1.75 -> 1.43 ms.
 
 // (2*(w>>9)+1) * 2^-24: exact, strictly inside (0,1): 1 + (w>>9) 2^-23 less 1 - 2^-24.
 DSANLS_DEV float uniform_open(uint32_t w) {
