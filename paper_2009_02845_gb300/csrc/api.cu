@@ -471,7 +471,9 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
     // one of the FP32 form's products (c_trans: stored transposed, split products only)
     auto product = [&](const GemmArgs &g, bool c_trans = false) {
         if (chained(h) || !split_gemm_supported(g.M, g.N, g.K)) {  // (A = X S of 7e8 columns)
-            launch_sgemm(g, s);
+            GemmArgs c = g;
+            c.beside = forked;
+            launch_sgemm(c, s);
             return;
         }
         launch_split_parts(g.B, g.ldb, g.b_kcontig, g.gb, g.N, g.K, h->Gparts, s);

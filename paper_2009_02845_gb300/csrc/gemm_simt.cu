@@ -191,8 +191,17 @@ void launch_sgemm(const GemmArgs &g, cudaStream_t s) {
     const int64_t small = ceil_div(g.M, ST) * ceil_div(g.N, ST) * splits;
     // large tiles from half a wave of them on, or where the small ones would be many waves
     // (2,429 x 100 from 200: 76 large tiles 14.6 us, 19.1 small; 4,096 x 64 from 1,000: 64
-    // large 49, 64 small; 1,665 x 100 from 100: 54 large 10.1, 8.5 small)
-    const int tile = mid >= 76 || (small > 6 * 152 && mid >= 16) ? MT : ST;
+    // large 49, 64 small; 1,665 x 100 from 100: 54 large 10.1, 8.5 small; over 361 .. 65,536 rows,
+    // ranks of 10 to 128 and K of 64 to 4,000 never slower than one 128-row tile at a time)
+    // Beside the Gram and the step size of a half-step (45 to 75 us of a few CTAs) the product is
+    // hidden as long as it is short, and the small tiles' many CTAs then only hold those up:
+    // coordinate descent on sampled columns, us per half-step with large / small tiles, 2,000
+    // rows: rank 10, K = 256 39.7 / 40.1, 350 41.6 / 40.6, 600 79 / 44; rank 31, 200 62.9 / 65.9, 420
+    // 65 / 68, 500 75 / 69; rank 64, 200 100 / 107, 500 106 / 116, 600 128 / 121; rank 100, 200 260 /
+    // 273, 700 280 / 306, 1,400 338 / 356.
+    const int64_t hidden = g.N <= 16 ? 300 : (g.N <= 32 ? 450 : (g.N <= 64 ? 550 : 2048));
+    const bool large = mid >= 76 || (small > 6 * 152 && mid >= 16) || (g.beside && g.K < hidden);
+    const int tile = large ? MT : ST;
     if (g.a_kcontig && g.b_kcontig) dispatch<true, true>(g, tile, s);
     else if (g.a_kcontig) dispatch<true, false>(g, tile, s);
     else if (g.b_kcontig) dispatch<false, true>(g, tile, s);

@@ -83,6 +83,7 @@ struct GemmArgs {
     float alpha;
     int splits;
     int64_t c_split_stride;
+    bool beside = false;  // launch_sgemm: runs beside a Gram and its step size on another stream
 };
 void launch_sgemm(const GemmArgs &g, cudaStream_t s);
 // out[i*ldo + j] = sum_{z<splits} part[z*stride + i*ldp + j], z ascending.
