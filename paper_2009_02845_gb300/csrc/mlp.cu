@@ -13,7 +13,8 @@
 // The weights used by the forward and backward passes are the fp32 master
 // weights rounded to bf16 (bf16 weights, fp32 accumulation); Adam updates the
 // fp32 masters.  Prediction's products run on tensor cores at binary32 accuracy
-// (gemm_split.cu: three-way bf16 splits; the weights are bf16 values, one part).
+// (gemm_split.cu: three-way bf16 splits; the weights are bf16 values, one part) but for the
+// one over the k columns of bn, too short for it.
 // Training's stay binary32 chains in the order of the rows (gemm_simt.cu, k_colsum): Adam
 // divides by the gradient's own size and the weights are rounded to bf16 after every step,
 // so a rounding difference of 1e-7 in a gradient moves the weights by 1e-5 to 1e-4 within
@@ -58,8 +59,7 @@ DSANLS_DEV void put_parts(const WeightParts &w, int64_t i, __nv_bfloat16 q) {
 // on theta first (the step and the rounding share one pass over the parameters).
 __global__ void k_adam_round(float *__restrict__ theta, float *__restrict__ m, float *__restrict__ v,
                              const float *__restrict__ g, int64_t n, float lr, float b1, float b2, float c1, float c2,
-                             float eps, float *__restrict__ wq, WeightParts w0, WeightParts w1, WeightParts w2,
-                             WeightParts w3) {
+                             float eps, float *__restrict__ wq, WeightParts w0, WeightParts w1, WeightParts w2) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float x = theta[i];
@@ -77,7 +77,6 @@ __global__ void k_adam_round(float *__restrict__ theta, float *__restrict__ m, f
     put_parts(w0, i, q);
     put_parts(w1, i, q);
     put_parts(w2, i, q);
-    put_parts(w3, i, q);
 }
 
 // per group: s_g and Gn_g; the first kernel of a pass clears the word that the pass's products raise
@@ -115,19 +114,21 @@ DSANLS_DEV int group_of(const int64_t *off, int ngroups, int64_t r) {
     return lo;
 }
 
-// one warp per row, one lane per column (k <= 32); the sum of squares in column order
+// W lanes per row, one per column (k <= W <= 32); the sum of squares in column order.  (A whole
+// warp for a row of 8 took 29 us for 57,556 rows, one thread 8.)
+template <int W>
 __global__ void __launch_bounds__(256) k_norm_rows(const float *__restrict__ b, int64_t rows, int k,
                                                    float *__restrict__ bn, float *__restrict__ beta) {
-    const int lane = threadIdx.x & 31;
-    const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (r >= rows) return;
-    const float x = lane < k ? b[r * k + lane] : 0.0f;
+    const int lane = threadIdx.x % W;
+    const int64_t r = (int64_t)blockIdx.x * (256 / W) + threadIdx.x / W;
+    const float x = r < rows && lane < k ? b[r * k + lane] : 0.0f;
     float ss = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        const float y = __shfl_sync(0xffffffffu, x, j);
+    for (int j = 0; j < W; ++j) {
+        const float y = __shfl_sync(0xffffffffu, x, j, W);
         ss = fmaf(y, y, ss);  // (zeros past k)
     }
+    if (r >= rows) return;
     float bt = sqrtf(ss / k);
     if (!(bt > 0.0f)) bt = 1.0f;
     if (lane == 0) beta[r] = bt;
@@ -354,7 +355,7 @@ void mlp_alloc(MlpState &st, int k, int h, int64_t max_rows, int max_groups) {
     al(st.loss, 2);  // the loss, then the error words
     st.err = reinterpret_cast<int *>(st.loss + 1);
     al(st.gf1, (int64_t)k * k); al(st.mu1, 1); al(st.off1, 2);
-    al(st.W1g, h * split_parts_ld((int64_t)k * k)); al(st.W1b, h * split_parts_ld(k)); al(st.W2, h * split_parts_ld(h));
+    al(st.W1g, h * split_parts_ld((int64_t)k * k)); al(st.W2, h * split_parts_ld(h));
     al(st.W3, k * split_parts_ld(h));
     // split-K partials of the Gram layer (batches of few groups)
     al(st.part, ceil_div((int64_t)k * k, 64) * std::min<int64_t>(max_groups, 19456) * h);
@@ -380,7 +381,7 @@ void mlp_free(MlpState &st) {
                     (void *)st.s, (void *)st.zg, (void *)st.dzg, (void *)st.bn, (void *)st.beta, (void *)st.z1,
                     (void *)st.h1, (void *)st.z2, (void *)st.h2, (void *)st.o, (void *)st.y, (void *)st.dout,
                     (void *)st.rowloss, (void *)st.loss, (void *)st.gf1, (void *)st.mu1, (void *)st.off1,
-                    (void *)st.W1g, (void *)st.W1b, (void *)st.W2, (void *)st.W3, (void *)st.part,
+                    (void *)st.W1g, (void *)st.W2, (void *)st.W3, (void *)st.part,
                     (void *)st.dz2})
         if (p) cudaFree(p);
     for (cudaStream_t t : st.side)
@@ -403,7 +404,6 @@ static void adam_round(MlpState &st, float lr, cudaStream_t s) {
     }
     k_adam_round<<<nblk(O.total), 256, 0, s>>>(st.theta, st.m, st.v, st.grad, O.total, lr, b1, b2, c1, c2, 1e-8f, st.wq,
                                                WeightParts{O.W1g, h, k * k, st.W1g},
-                                               WeightParts{O.W1b, h, k, st.W1b},
                                                WeightParts{O.W2, h, h, st.W2},
                                                WeightParts{O.W3, k, h, st.W3});
     DSANLS_LAUNCH_CHECK();
@@ -433,12 +433,16 @@ void mlp_forward(MlpState &st, const float *G, const float *mu, const int64_t *o
         launch_split_gemm(SplitGemm{ngroups, h, kk, st.Gn, kk, true, nullptr, st.W1g, 1, st.zg, h, false, 1.0f, st.part,
                                     ngroups <= 19456 ? MLP_MAX_SPLITS : 1},
                           err, s);
-    k_norm_rows<<<(unsigned)ceil_div(rows, 8), 256, 0, s>>>(b, rows, k, st.bn, st.beta);
-    DSANLS_LAUNCH_CHECK();
-    if (training)
-        chain(rows, h, k, st.bn, k, true, W + O.W1b, k, true, st.z1, h, s);
+    if (k <= 8)
+        k_norm_rows<8><<<(unsigned)ceil_div(rows, 32), 256, 0, s>>>(b, rows, k, st.bn, st.beta);
+    else if (k <= 16)
+        k_norm_rows<16><<<(unsigned)ceil_div(rows, 16), 256, 0, s>>>(b, rows, k, st.bn, st.beta);
     else
-        times_weights(rows, h, k, st.bn, st.W1b, st.z1, err, s);
+        k_norm_rows<32><<<(unsigned)ceil_div(rows, 8), 256, 0, s>>>(b, rows, k, st.bn, st.beta);
+    DSANLS_LAUNCH_CHECK();
+    // (K = k <= 32: the CTAs of the split product have a block or two each; 57,556 x 64 from 8
+    // 52 us there, 20 here, and 1,000 .. 57,556 x 256 from 32 the same)
+    chain(rows, h, k, st.bn, k, true, W + O.W1b, k, true, st.z1, h, s);
     k_layer1_finish<<<(unsigned)ceil_div(rows, ACT_ROWS), (unsigned)std::min(256, (h + 31) / 32 * 32), 0, s>>>(
         st.z1, st.h1, st.zg, W + O.b1, off, ngroups, rows, h);
     DSANLS_LAUNCH_CHECK();

@@ -28,7 +28,7 @@ struct MlpState {
     // such a prediction until a synchronising call has reported it (both behind the loss)
     int *err = nullptr;
     // the rounded weights as second operands of prediction's products
-    __nv_bfloat16 *W1g = nullptr, *W1b = nullptr, *W2 = nullptr, *W3 = nullptr;
+    __nv_bfloat16 *W1g = nullptr, *W2 = nullptr, *W3 = nullptr;
     float *part = nullptr;  // split-K partials
     // training (from the first step on): dz2, and side streams with their events
     float *dz2 = nullptr;
