@@ -748,6 +748,11 @@ void make_reduced_copies(dsanls_ctx *h) {
         launch_copy_cast_bf16(h->M, h->m * h->n, h->Mb, s);
         launch_copy_cast_bf16(h->MT, h->m * h->n, h->MTb, s);
     }
+    if (h->opt.precision == DSANLS_PREC_FP32 && !fp32_split(h))  // (another order or solver: nothing reads them)
+        for (int a = 0; a < 3; ++a) {
+            dfree(h->M3[a]);
+            dfree(h->MT3[a]);
+        }
     if (fp32_split(h) && !h->M3[0]) {
         for (int a = 0; a < 3; ++a) {
             dalloc(h->M3[a], h->m * h->n);
