@@ -315,7 +315,8 @@ void column_sums(const float *X, const int64_t *off, int nseg, int64_t rows, int
     DSANLS_LAUNCH_CHECK();
 }
 
-constexpr int MLP_MAX_SPLITS = 64;  // of the Gram layer's product
+// The Gram layer's product: most slices of its K, for batches of at most so many subproblems
+constexpr int MLP_MAX_SPLITS = 64, MLP_SPLIT_GROUPS = 19456;
 
 }  // namespace
 
@@ -357,8 +358,12 @@ void mlp_alloc(MlpState &st, int k, int h, int64_t max_rows, int max_groups) {
     al(st.gf1, (int64_t)k * k); al(st.mu1, 1); al(st.off1, 2);
     al(st.W1g, h * split_parts_ld((int64_t)k * k)); al(st.W2, h * split_parts_ld(h));
     al(st.W3, k * split_parts_ld(h));
-    // split-K partials of the Gram layer (batches of few groups)
-    al(st.part, ceil_div((int64_t)k * k, 64) * std::min<int64_t>(max_groups, 19456) * h);
+    // split-K partials of the Gram layer: the most that its plan takes for any number of groups
+    // (at most 10 MB: from 9,728 groups on it does not split)
+    int64_t most = 0;
+    for (int64_t g = 1; g <= std::min<int64_t>(max_groups, MLP_SPLIT_GROUPS); ++g)
+        most = std::max(most, split_gemm_plan(g, h, (int64_t)k * k, MLP_MAX_SPLITS).part_elems);
+    al(st.part, most);
     DSANLS_CUDA(cudaMemset(st.loss, 0, 2 * sizeof(double)));
     DSANLS_CUDA(cudaMemset(st.m, 0, P * sizeof(float)));
     DSANLS_CUDA(cudaMemset(st.v, 0, P * sizeof(float)));
@@ -431,7 +436,7 @@ void mlp_forward(MlpState &st, const float *G, const float *mu, const int64_t *o
         chain(ngroups, h, kk, st.Gn, kk, true, W + O.W1g, kk, true, st.zg, h, s);
     else
         launch_split_gemm(SplitGemm{ngroups, h, kk, st.Gn, kk, true, nullptr, st.W1g, 1, st.zg, h, false, 1.0f, st.part,
-                                    ngroups <= 19456 ? MLP_MAX_SPLITS : 1},
+                                    ngroups <= MLP_SPLIT_GROUPS ? MLP_MAX_SPLITS : 1},
                           err, s);
     if (k <= 8)
         k_norm_rows<8><<<(unsigned)ceil_div(rows, 32), 256, 0, s>>>(b, rows, k, st.bn, st.beta);
