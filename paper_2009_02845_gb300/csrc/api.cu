@@ -472,7 +472,7 @@ void half_step(dsanls_ctx *h, int side, cudaStream_t s, PhaseEvents *pe = nullpt
     auto product = [&](const GemmArgs &g, bool c_trans = false) {
         if (chained(h) || !split_gemm_supported(g.M, g.N, g.K)) {  // (A = X S of 7e8 columns)
             GemmArgs c = g;
-            c.beside = forked;
+            c.beside = forked && h->sketch == DSANLS_SKETCH_SUBSAMPLE;  // (one product; two in a row outlast the Gram)
             launch_sgemm(c, s);
             return;
         }
