@@ -48,10 +48,10 @@
 //                  64 (from L2).
 // What bounds it: HBM needs 1,515 cycles per tile, the products 1,280 (k <= 64), the
 // epilogue's issue slots about 1,400.  Measured, with the parts and the final sum, 65,536 x
-// 16,384 with k = 64: 1.24 ms (11.6 in FP64) = 3.5 TB/s, and
-// 2.56 where the columns are balanced in a second pass; k = 100 1.78.  The epilogue's arithmetic
-// bounds it (0.99 ms without): it runs two columns to an instruction (1.37 ms with one), reads M
-// before it waits for the products and its accumulators with one wait (1.35 otherwise).
+// 16,384 with k = 64: 1.21 ms (11.6 in FP64) = 3.6 TB/s, 2.50 where the columns are balanced in
+// a second pass; k = 100 1.77.  The epilogue's arithmetic bounds it (0.99 ms without): it runs
+// two columns to an instruction (1.37 ms with one), reads M before it waits for the products
+// and its accumulators with one wait (1.35 otherwise).
 #include <cuda.h>
 
 #include <algorithm>
@@ -372,10 +372,13 @@ __global__ void __launch_bounds__(256) k_column_max(const float *__restrict__ U,
 }
 
 // The four parts of the rows of U (blocks 0 .. ublocks-1) and V (the rest) on each row's grid,
-// out[p][row][ldk], prows rows per part (zero past the last); one warp per row.  A row whose
-// largest entry is not in [2^-90, 2^100], or not finite, becomes NaN: the result is then not
-// finite.  Each block's sum of (nonzeros) 4^e goes to sums[b].
-// With cmax the columns are balanced first (a column that is zero in either factor is dropped).
+// out[p][row][ldk], prows rows per part (zero past the last); one warp per row, the next row's
+// entries on their way.  A row whose largest entry is not in [2^-90, 2^100], or not finite,
+// becomes NaN: the result is then not finite.  Each block's sum of (nonzeros) 4^e goes to
+// sums[b]; a warp keeps its own as acc 4^ref (in FP64 the row's few operations were two thirds
+// of the kernel).  With cmax the columns are balanced first (a column that is zero in either
+// factor is dropped).  NC: columns per lane, k <= 32 NC.
+template <int NC>
 __global__ void __launch_bounds__(256)
     k_parts_grid(const float *__restrict__ U, const float *__restrict__ V, int64_t m, int64_t n, int k, int64_t ldk,
                  int64_t ur, int64_t vr, __nv_bfloat16 *__restrict__ parts, int ublocks,
@@ -387,42 +390,51 @@ __global__ void __launch_bounds__(256)
     __nv_bfloat16 *out = parts + (is_v ? RT_PARTS * ur * ldk : 0);
     const int blk = (int)blockIdx.x - (is_v ? ublocks : 0), nblk = is_v ? (int)gridDim.x - ublocks : ublocks;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float f[4] = {1.0f, 1.0f, 1.0f, 1.0f}, f2[4] = {1.0f, 1.0f, 1.0f, 1.0f};  // the column's factor in two steps
-    if (cmax) {
+    float f[NC], f2[NC];  // the column's factor in two steps
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int c = lane + 32 * u;
-            if (c >= k) break;
-            const uint32_t a = cmax[c], b = cmax[RT_COLS + c];
-            const int t = ((int)(b >> 23) - (int)(a >> 23)) >> 1, e = is_v ? -t : t;  // |t| <= 127
-            f[u] = a && b ? __int_as_float((127 + (e >> 1)) << 23) : 0.0f;
-            f2[u] = __int_as_float((127 + e - (e >> 1)) << 23);
-        }
+    for (int u = 0; u < NC; ++u) {
+        const int c = lane + 32 * u;
+        f[u] = f2[u] = 1.0f;
+        if (!cmax || c >= k) continue;
+        const uint32_t a = cmax[c], b = cmax[RT_COLS + c];
+        const int t = ((int)(b >> 23) - (int)(a >> 23)) >> 1, e = is_v ? -t : t;  // |t| <= 127
+        f[u] = a && b ? __int_as_float((127 + (e >> 1)) << 23) : 0.0f;
+        f2[u] = __int_as_float((127 + e - (e >> 1)) << 23);
     }
-    double sum = 0.0;
-    for (int64_t r = (int64_t)blk * 8 + warp; r < prows; r += (int64_t)nblk * 8) {
-        float z[4], mx = 0.0f;
-        bool finite = true;
-        int nz = 0;
+    const int64_t step = (int64_t)nblk * 8;
+    float acc = 0.0f, next[NC];
+    int ref = -128;
+    auto load = [&](int64_t r) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int c = lane + 32 * u;
-            z[u] = r < rows && c < k ? X[r * k + c] : 0.0f;
-            finite = finite && fabsf(z[u]) <= 3.402823466e38f;
-            z[u] = __fmul_rn(__fmul_rn(z[u], f[u]), f2[u]);
-            finite = finite && fabsf(z[u]) <= 3.402823466e38f;
-            mx = fmaxf(mx, fabsf(z[u]));
-            nz += __popc(__ballot_sync(0xffffffffu, z[u] != 0.0f));
+        for (int u = 0; u < NC; ++u) next[u] = r < rows && lane + 32 * u < k ? X[r * k + lane + 32 * u] : 0.0f;
+    };
+    load((int64_t)blk * 8 + warp);
+    for (int64_t r = (int64_t)blk * 8 + warp; r < prows; r += step) {
+        float z[NC];
+        unsigned bits = 0, nz = 0;
+#pragma unroll
+        for (int u = 0; u < NC; ++u) {
+            z[u] = cmax ? __fmul_rn(__fmul_rn(next[u], f[u]), f2[u]) : next[u];
+            bits = max(bits, __float_as_uint(z[u]) & 0x7fffffffu);  // (NaN above Inf above all numbers)
+            nz += z[u] != 0.0f;
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        const bool bad = !__all_sync(0xffffffffu, finite) || (mx > 0.0f && (mx < 0x1p-90f || mx > 0x1p100f));
+        load(r + step);
+        bits = __reduce_max_sync(0xffffffffu, bits);
+        nz = __reduce_add_sync(0xffffffffu, nz);
+        const float mx = __uint_as_float(bits);
+        const bool bad = bits && !(mx >= 0x1p-90f && mx <= 0x1p100f);
         // e: 2^e above every entry; rounding to a multiple of q by adding and subtracting 1.5 2^23 q
-        const int e = mx > 0.0f && !bad ? (int)((__float_as_uint(mx) >> 23) & 255) - 126 : 0;
-        if (mx > 0.0f) sum += ldexp((double)nz, 2 * e);
+        const int e = bits && !bad ? (int)(bits >> 23) - 126 : 0;
+        if (bits) {
+            if (e > ref) {
+                acc = ref - e < -63 ? 0.0f : acc * __int_as_float((127 + 2 * (ref - e)) << 23);
+                ref = e;
+            }
+            if (e - ref >= -63) acc += (float)nz * __int_as_float((127 + 2 * (e - ref)) << 23);
+        }
         const float c1 = __int_as_float((127 + e + 15) << 23) * 1.5f;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < NC; ++u) {
             const int c = lane + 32 * u;
             if (c >= k) break;
             __nv_bfloat16 *o = out + r * ldk + c;
@@ -436,7 +448,7 @@ __global__ void __launch_bounds__(256)
             }
         }
     }
-    if (lane == 0) red[warp] = sum;
+    if (lane == 0) red[warp] = ldexp((double)acc, 2 * ref);
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
@@ -445,31 +457,29 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// out[0] = the squared residual, out[1] = E^2 (the head of this file); fixed orders
-__global__ void __launch_bounds__(256)
+// out[0] = the squared residual, out[1] = E^2 (the head of this file): three sums in fixed
+// orders, eight warps each (one warp's shuffles for all three took 2 us more)
+__global__ void __launch_bounds__(768)
     k_residual_sum(const double *__restrict__ part, int np, const double *__restrict__ sums, int ublocks, int vblocks,
                    double m, double n, double k, double *__restrict__ out) {
-    __shared__ double red[3][8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double v[3] = {0.0, 0.0, 0.0};  // the residual, U's and V's nz 4^e
-    for (int i = threadIdx.x; i < np; i += 256) v[0] += part[i];
-    for (int i = threadIdx.x; i < ublocks; i += 256) v[1] += sums[i];
-    for (int i = threadIdx.x; i < vblocks; i += 256) v[2] += sums[ublocks + i];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-        if (lane == 0) red[q][warp] = v[q];
-    }
+    __shared__ double red[24];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp >> 3;  // the residual, U's and V's nz 4^e
+    const double *x = q == 0 ? part : (q == 1 ? sums : sums + ublocks);
+    const int len = q == 0 ? np : (q == 1 ? ublocks : vblocks);
+    double v = 0.0;
+#pragma unroll 4
+    for (int i = threadIdx.x & 255; i < len; i += 256) v += x[i];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[warp] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t[3];
-        for (int q = 0; q < 3; ++q) {
-            t[q] = 0.0;
-            for (int w = 0; w < 8; ++w) t[q] += red[q][w];
-        }
+    if (warp > 0) return;
+    v = lane < 24 ? red[lane] : 0.0;
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);  // eight lanes to a sum
+    const double u4 = __shfl_sync(0xffffffffu, v, 8), v4 = __shfl_sync(0xffffffffu, v, 16);
+    if (lane == 0) {
         const double under = k * 0x1p-125;
-        out[0] = t[0];
-        out[1] = 26.0 * 0x1p-72 * t[1] * t[2] + m * n * under * under;
+        out[0] = v;
+        out[1] = 26.0 * 0x1p-72 * u4 * v4 + m * n * under * under;
     }
 }
 
@@ -517,7 +527,8 @@ void launch_dense_residual_tc(const float *M, int64_t ld, const float *U, const 
         k_column_max<<<dim3((unsigned)std::max(ublocks, vblocks), 2), 256, 0, s>>>(U, V, m, n, k, cmax);
         DSANLS_LAUNCH_CHECK();
     }
-    k_parts_grid<<<(unsigned)(ublocks + vblocks), 256, 0, s>>>(U, V, m, n, k, ldk, ur, vr, up, ublocks,
+    const auto parts_kernel = k <= 32 ? k_parts_grid<1> : (k <= 64 ? k_parts_grid<2> : k_parts_grid<4>);
+    parts_kernel<<<(unsigned)(ublocks + vblocks), 256, 0, s>>>(U, V, m, n, k, ldk, ur, vr, up, ublocks,
                                                                balance ? cmax : nullptr, sums);
     DSANLS_LAUNCH_CHECK();
     CUtensorMap mm_map, mu, mv;
@@ -530,7 +541,7 @@ void launch_dense_residual_tc(const float *M, int64_t ld, const float *U, const 
         residual_launch<1>(mm_map, mu, mv, m, n, k, mm, work, grid, err, s);
     else
         residual_launch<2>(mm_map, mu, mv, m, n, k, mm, work, grid, err, s);
-    k_residual_sum<<<1, 256, 0, s>>>(work, grid, sums, ublocks, vblocks, (double)m, (double)n, (double)k, out);
+    k_residual_sum<<<1, 768, 0, s>>>(work, grid, sums, ublocks, vblocks, (double)m, (double)n, (double)k, out);
     DSANLS_LAUNCH_CHECK();
 }
 
