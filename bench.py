@@ -526,9 +526,16 @@ def run_ours(args, w):
             bound, peak, unit = "hbm", peaks["hbm_gbs"], "GB/s"
             kernel_key = "tc_skinny" if prec == pkg.BF16 else "tc_skinny_fp8"
             peak_note = "hbm_gbs of %s" % peak_src
+        elif args.solver == "pgd":
+            # FP32 on tensor cores: X read once as binary32 (split on the way), the parts of the
+            # K x k factor (6 bytes per entry)
+            bytes_ = [4.0 * (m * n + m * k) + 6.0 * k * n, 4.0 * (n * m + n * k) + 6.0 * k * m]
+            achieved = sum(bytes_) / (sum(prod_ms) / 1000.0) / 1e9
+            bound, peak, unit, kernel_key = "hbm", peaks["hbm_gbs"], "GB/s", "split_gemm"
+            peak_note = "hbm_gbs of %s" % peak_src
         elif m % 8 == 0 and n % 8 == 0 and dense_sketch:
-            # FP32 on tensor cores: the streaming product reads the three bf16 parts of X
-            # (6 bytes per entry) and the parts of P^T
+            # Alg. 3: the streaming product reads the three bf16 parts of X (6 bytes per entry)
+            # and the parts of P^T
             bytes_ = [6.0 * (m * n + k * n) + 4.0 * m * k, 6.0 * (n * m + k * m) + 4.0 * n * k]
             achieved = sum(bytes_) / (sum(prod_ms) / 1000.0) / 1e9
             bound, peak, unit, kernel_key = "hbm", peaks["hbm_gbs"], "GB/s", "tc_skinny_split3"
@@ -557,6 +564,10 @@ def run_ours(args, w):
             bound, peak, unit, kernel_key = "tensor", peaks["bf16_tflops"] / 6.0, "TFLOP/s", "tc_gemm_split3"
             peak_note = ("bf16_tflops (burst) of %s / 6: A = X S as six bf16 products of three-way splits "
                          "(algorithmic FP32 flops 2 rows K d per half)" % peak_src)
+        elif args.solver == "pgd":  # the same products, X split on the way
+            bound, peak, unit, kernel_key = "tensor", peaks["bf16_tflops"] / 6.0, "TFLOP/s", "split_gemm"
+            peak_note = ("bf16_tflops (burst) of %s / 6: A = X S as six bf16 products of three-way splits "
+                         "(algorithmic FP32 flops 2 rows K d per half)" % peak_src)
         else:
             bound, peak, unit, kernel_key = "alu", FP32_SIMT_PEAK_TFLOPS, "TFLOP/s", "sgemm_simt"
             peak_note = "FP32 CUDA-core peak 152 SMs x 128 lanes x 2 FLOP x 2.07 GHz"
@@ -565,14 +576,15 @@ def run_ours(args, w):
         bytes_ = [4.0 * (m * d + d * k) + 4.0 * m * k, 4.0 * (n * d_v + d_v * k) + 4.0 * n * k]
         prod_ms = [p["rhs"] for p in phases]
         achieved = sum(bytes_) / (sum(prod_ms) / 1000.0) / 1e9
-        bound, peak, unit, kernel_key = "hbm", peaks["hbm_gbs"], "GB/s", "sgemm_simt_gather"
+        bound, peak, unit = "hbm", peaks["hbm_gbs"], "GB/s"
+        kernel_key = "split_gemm_gather" if args.solver == "pgd" else "sgemm_simt_gather"
         peak_note = "hbm_gbs of %s" % peak_src
     else:
         # sparse subsampling: the row update forms the right-hand side of the sampled entries
         # itself -- it reads and writes Z (8 bytes per element; 4 with bf16 factors), the row
         # pointers (8 bytes per row) and sampled entries (8 bytes each; nnz d / K expected) of
         # the sub-CSR and the d sampled rows of the other factor (R only for the few rows of
-        # more than 64 entries, not counted)
+        # more than 16 entries, not counted)
         zb = 4.0 if prec == pkg.BF16 else 8.0
         es = 2.0 if prec == pkg.BF16 else 4.0
         nnz = float(len(M[1]))

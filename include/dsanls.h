@@ -87,7 +87,9 @@ extern "C" {
  * of the product), otherwise on CUDA cores in binary32. */
 
 /* ---- arithmetic of the sketched products A = M S and R = A B^T -------- */
-#define DSANLS_PREC_FP32 0    /* binary32 operands, products at binary32 accuracy */
+#define DSANLS_PREC_FP32 0    /* binary32 operands, products at binary32 accuracy
+                                 (entries of 1e-33 .. 3.39e38; smaller ones lose
+                                 bits on tensor cores, larger ones overflow)      */
 #define DSANLS_PREC_BF16 1    /* bf16 operands, fp32 accumulation (tcgen05)       */
 #define DSANLS_PREC_FP8 2     /* fp8 E4M3 M (one scale per 128-row block) and S
                                  (entries N(0,1), 1/sqrt(d) applied to the fp32

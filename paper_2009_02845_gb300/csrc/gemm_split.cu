@@ -1,12 +1,14 @@
 // Binary32-accurate GEMM on tcgen05 tensor cores from a binary32 first operand (the
 // FP32 form's products: A = X S, R = A B^T, the sampled R = c^2 X[:, J] Y[J, :],
-// B = Y^T S, and the warm start's network).
+// B = Y^T S, and the wide products of the warm start's prediction).
 //
 // Every element is three bf16 parts, z = h + m + l (split3), and the six products
 // whose parts' orders add to at most 2 are taken; the dropped ones are of order 2^-24
-// of the product.  The second operand's parts are made beforehand (it is small or
-// used by every row tile); the first operand's on its way through shared memory, so a
-// large matrix is read once, as binary32, and no split copy of it is kept.  The parts
+// of the product.  (The parts are bf16 values: below about 1e-33 an entry's third one is
+// rounded or lost, between 3.39e38 and the largest binary32 its first is infinite.)  The
+// second operand's parts are made beforehand (it is small or used by every row tile); the
+// first operand's on its way to tensor memory, so a large matrix is read once, as binary32,
+// and no split copy of it is kept.  The parts
 // of the second operand lie side by side (BN columns each), so one K step takes the
 // MMAs A_h x [B_h | B_m | B_l], A_m x [B_h | B_m], A_l x B_h (N = 3, 2, 1 BN; an MMA of
 // N < 96 costs as much as one of 96) into three column blocks of tensor memory by
