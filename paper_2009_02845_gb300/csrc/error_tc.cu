@@ -48,10 +48,11 @@
 //                  64 (from L2).
 // What bounds it: HBM needs 1,515 cycles per tile, the products 1,280 (k <= 64), the
 // epilogue's issue slots about 1,400.  Measured, with the parts and the final sum, 65,536 x
-// 16,384 with k = 64: 1.21 ms (11.6 in FP64) = 3.6 TB/s, 2.50 where the columns are balanced in
-// a second pass; k = 100 1.77.  The epilogue's arithmetic bounds it (0.99 ms without): it runs
-// two columns to an instruction (1.37 ms with one), reads M before it waits for the products
-// and its accumulators with one wait (1.35 otherwise).
+// 16,384 with k = 64: 1.17 ms (11.6 in FP64) = 3.7 TB/s, about twice that where the columns are
+// balanced in a second pass; k = 100, whose products take 2,560 cycles a tile, 1.81.  The
+// epilogue's arithmetic and the latency of its loads bound it: it runs two columns to an
+// instruction (1.46 ms with one), reads M before it waits for the products and its
+// accumulators with one wait (1.35 otherwise).
 #include <cuda.h>
 
 #include <algorithm>
@@ -192,54 +193,55 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
         const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16) + 16 * cg;
         const float sc = __int_as_float((127 - rt_exponent(*mm, (double)m * (double)n)) << 23);
         const uint64_t scale = rt_pair(sc, sc);
-        for (int i = 0; i < nt; ++i) {
-            const int c = 2 * i + (cg >> 1), slot = c % MST, buf = i & 1;
-            bool ok = role_wait(&tail->mfull[slot], (c / MST) & 1, abort, wait.ns);
-            if (!__all_sync(0xffffffffu, ok)) break;
-            const float4 *row = reinterpret_cast<const float4 *>(mp + slot * RT_CHUNK_BYTES) + r * (RT_CHUNK / 4);
-            float4 v[4];
+        // (a loop of its own for the carry: under a condition in this one its FP64 conversions and
+        // additions run for every tile, 2,000 cycles of the FP64 pipe: 1.21 ms, k = 31 17 % more)
+        bool ok = true;
+        for (int i0 = 0; ok && i0 < nt; i0 += RT_CARRY) {
+            const int i1 = min(nt, i0 + RT_CARRY);
+            for (int i = i0; i < i1; ++i) {
+                const int c = 2 * i + (cg >> 1), slot = c % MST, buf = i & 1;
+                ok = role_wait(&tail->mfull[slot], (c / MST) & 1, abort, wait.ns);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                const float4 *row = reinterpret_cast<const float4 *>(mp + slot * RT_CHUNK_BYTES) + r * (RT_CHUNK / 4);
+                float4 v[4];
 #pragma unroll
-            for (int p = 0; p < 4; ++p) v[p] = row[(4 * (cg & 1) + p) ^ (r & 7)];
-            if (MST == 2) {  // a ring of one tile: the next one's copy under this one's products (k = 100
-                __syncwarp();  // 1.79 ms, 2.44 with the arrival below; k = 64, three tiles, 1.30 and 1.23)
-                if (lane == 0) mbar_arrive(&tail->mempty[slot]);
-            }
-            ok = role_wait(&tail->dfull[buf], (i >> 1) & 1, abort, wait.ns);
-            if (!__all_sync(0xffffffffu, ok)) break;
-            fence_after();
-            uint32_t d[16], d1[16], d2[16], d3[16];
-            uint64_t x[8];
-            tmem_ld16(tl + buf * RT_DSET, d);
-            tmem_ld16(tl + buf * RT_DSET + RT_BN, d1);
-            tmem_ld16(tl + buf * RT_DSET + 2 * RT_BN, d2);
-            tmem_ld16(tl + buf * RT_DSET + 3 * RT_BN, d3);
-            tmem_ld_wait();
+                for (int p = 0; p < 4; ++p) v[p] = row[(4 * (cg & 1) + p) ^ (r & 7)];
+                __syncwarp();  // (the next copy runs under these products: with a ring of one tile, k = 100,
+                if (lane == 0) mbar_arrive(&tail->mempty[slot]);  // 2.44 ms when released below, 1.79 here)
+                ok = role_wait(&tail->dfull[buf], (i >> 1) & 1, abort, wait.ns);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                fence_after();
+                uint32_t d[16], d1[16], d2[16], d3[16];
+                uint64_t x[8];
+                tmem_ld16(tl + buf * RT_DSET, d);
+                tmem_ld16(tl + buf * RT_DSET + RT_BN, d1);
+                tmem_ld16(tl + buf * RT_DSET + 2 * RT_BN, d2);
+                tmem_ld16(tl + buf * RT_DSET + 3 * RT_BN, d3);
+                tmem_ld_wait();
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                x[e] = rt_add(rt_pair(d2[2 * e], d2[2 * e + 1]), rt_pair(d3[2 * e], d3[2 * e + 1]));
-            fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&tail->dempty[buf]);
-                if (MST > 2) mbar_arrive(&tail->mempty[slot]);
-            }
+                for (int e = 0; e < 8; ++e)
+                    x[e] = rt_add(rt_pair(d2[2 * e], d2[2 * e + 1]), rt_pair(d3[2 * e], d3[2 * e + 1]));
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tail->dempty[buf]);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float4 w = v[e >> 1];
-                const uint64_t me = (e & 1) ? rt_pair(w.z, w.w) : rt_pair(w.x, w.y);
-                const uint64_t r1 = rt_sub(rt_sub(me, rt_pair(d[2 * e], d[2 * e + 1])), rt_pair(d1[2 * e], d1[2 * e + 1]));
-                const uint64_t res = rt_mul(rt_sub(r1, x[e]), scale);
-                const uint64_t p = rt_mul(res, res), pe = rt_fma(res, res, p ^ 0x8000000080000000ull);
-                // (hi, lo) += p + pe: columns past n and rows past m have a residual of zero
-                const uint64_t s = rt_add(hi, p), t = rt_sub(s, hi);
-                const uint64_t se = rt_add(rt_sub(hi, rt_sub(s, t)), rt_sub(p, t));
-                hi = s;
-                lo = rt_add(lo, rt_add(se, pe));
+                for (int e = 0; e < 8; ++e) {
+                    const float4 w = v[e >> 1];
+                    const uint64_t me = (e & 1) ? rt_pair(w.z, w.w) : rt_pair(w.x, w.y);
+                    const uint64_t r1 = rt_sub(rt_sub(me, rt_pair(d[2 * e], d[2 * e + 1])), rt_pair(d1[2 * e], d1[2 * e + 1]));
+                    const uint64_t res = rt_mul(rt_sub(r1, x[e]), scale);
+                    const uint64_t p = rt_mul(res, res), pe = rt_fma(res, res, p ^ 0x8000000080000000ull);
+                    // (hi, lo) += p + pe: columns past n and rows past m have a residual of zero
+                    const uint64_t s = rt_add(hi, p), t = rt_sub(s, hi);
+                    const uint64_t se = rt_add(rt_sub(hi, rt_sub(s, t)), rt_sub(p, t));
+                    hi = s;
+                    lo = rt_add(lo, rt_add(se, pe));
+                }
             }
-            if (i % RT_CARRY == RT_CARRY - 1) {
-                sum += rt_total(hi, lo);
-                hi = lo = 0;
-            }
+            sum += rt_total(hi, lo);
+            hi = lo = 0;
         }
     } else if (warp == RT_EW) {
         if (lane == 0) {
@@ -335,7 +337,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1)
                 mbar_wait(&tail->bfull[b % RT_BST], (b / RT_BST) & 1, wait.ns);
         }
     }
-    double v = sum + rt_total(hi, lo);
+    double v = sum;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (warp < RT_EW && lane == 0) tail->red[warp] = v;
     fence_before();
