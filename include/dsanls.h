@@ -189,8 +189,11 @@ int dsanls_step(dsanls_t h, int32_t outer_iters);
  * (eq. sketched_u), side 1 updates V (eq. sketched_v) using the current U. */
 int dsanls_half_step(dsanls_t h, int32_t side);
 
-/* ||M - U V^T||_F / ||M||_F of the current factors (Section 5.1), FP64
- * accumulation.  Synchronises; reports pending asynchronous errors. */
+/* ||M - U V^T||_F / ||M||_F of the current factors (Section 5.1).  Dense M: on
+ * tensor cores where a bound computed with the result leaves it within 1e-6 of
+ * itself or 2e-9 (absolute) of its FP64 value, else with binary32 inner
+ * products and FP64 residuals.  Sparse M: FP64 accumulation.  Synchronises;
+ * reports pending asynchronous errors. */
 int dsanls_rel_error(dsanls_t h, double *out);
 
 /* Copy U (m x k) and V (n x k) out; either may be NULL.  Synchronises. */

@@ -167,8 +167,8 @@ template <int BN, bool AK, int NPB>
 __global__ void __launch_bounds__(SgCfg<BN>::THREADS, 1)
     k_split_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int64_t M,
                  int64_t N, int64_t K, const float *__restrict__ A, int64_t lda, const int32_t *__restrict__ gather,
-                 int tma, int avec, WaitSwitch wait, float *__restrict__ C, int64_t ldm, int64_t ldn, float alpha, int kb_per_split,
-                 int64_t c_split_stride, int *__restrict__ err) {
+                 int tma, int avec, WaitSwitch wait, float *__restrict__ C, int64_t ldm, int64_t ldn, float alpha,
+                 int kb_per_split, int64_t c_split_stride, int *__restrict__ err) {
     using Cfg = SgCfg<BN>;
     constexpr int CW = Cfg::CW, AW = Cfg::AW, NSET = Cfg::NSET, FLUSH = Cfg::FLUSH, RAW = Cfg::RAW;
     constexpr int BST = Cfg::BST, AST = Cfg::AST, BPART = BN * 128;
@@ -503,8 +503,9 @@ void sg_launch(const SplitGemm &g, float *dst, int64_t ldm, int64_t ldn, const S
     else if (tma)
         encode_f32_map(&ma, g.A, g.K, g.M, g.lda, SG_BM, SG_RK, false);
     const auto kernel = g.a_kcontig ? k_split_gemm<BN, true, NPB> : k_split_gemm<BN, false, NPB>;
-    kernel<<<grid, SgCfg<BN>::THREADS, sg_smem<BN>(), s>>>(ma, mb, g.M, g.N, g.K, g.A, g.lda, g.gather, tma, avec, wait_switch(), dst,
-                                                           ldm, ldn, g.alpha, p.kb_per_split, g.M * g.N, err);
+    kernel<<<grid, SgCfg<BN>::THREADS, sg_smem<BN>(), s>>>(ma, mb, g.M, g.N, g.K, g.A, g.lda, g.gather, tma, avec,
+                                                           wait_switch(), dst, ldm, ldn, g.alpha, p.kb_per_split,
+                                                           g.M * g.N, err);
     DSANLS_LAUNCH_CHECK();
 }
 

@@ -530,7 +530,8 @@ void launch_update_tc_any(ZT *Z, const float *R, int64_t rows, int k, const floa
     if (ntiles / grid >= (1ll << 28)) throw ArgError{"launch_update_tc: too many rows"};
     const size_t smem = fixed + sh.nz * (size_t)sh.zbytes;
     const auto kern = k % 4 == 0 ? k_update_tc<ZT, SPR, true> : k_update_tc<ZT, SPR, false>;
-    kern<<<(unsigned)grid, 32 * (UPD_SPLIT + sh.na * (UPD_STEPS / upd_groups<ZT>()) + 2), smem, s>>>(Z, R, rows, sh, Gf, kp, scal, bound, flag, sub, wait_switch());
+    const int threads = 32 * (UPD_SPLIT + sh.na * (UPD_STEPS / upd_groups<ZT>()) + 2);
+    kern<<<(unsigned)grid, threads, smem, s>>>(Z, R, rows, sh, Gf, kp, scal, bound, flag, sub, wait_switch());
     DSANLS_LAUNCH_CHECK();
 }
 
