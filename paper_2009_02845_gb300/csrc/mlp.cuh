@@ -71,4 +71,5 @@ struct dsanls_mlp_ctx {
     dsanls::MlpState st;
     int device = 0;
     cudaStream_t own_stream = nullptr;
+    bool predicted = false;  // a prediction was queued: its error word may be raised
 };

@@ -46,6 +46,7 @@ int check_batch(const dsanls_mlp_ctx *m, const float *G, const float *mu, const 
 // after a synchronisation: the timeout that a prediction since the last report left, if any
 int pending_prediction(dsanls_mlp_ctx *m) {
     int failed = 0;
+    if (!m->predicted) return DSANLS_OK;
     DSANLS_CUDA(cudaMemcpy(&failed, m->st.err + 1, sizeof failed, cudaMemcpyDeviceToHost));
     if (!failed) return DSANLS_OK;
     DSANLS_CUDA(cudaMemset(m->st.err + 1, 0, sizeof(int)));
@@ -122,6 +123,7 @@ int dsanls_mlp_predict(dsanls_mlp_t m, const float *G, const float *mu, const in
     if (int rc = check_batch(m, G, mu, group_off, ngroups, b, rows)) return rc;
     return mguard([&]() {
         cudaStream_t s = (cudaStream_t)stream;
+        m->predicted = true;
         mlp_forward(m->st, G, mu, group_off, ngroups, b, rows, false, m->st.err, s);
         mlp_unscale(m->st, group_off, ngroups, rows, x_out, s);
         return DSANLS_OK;
